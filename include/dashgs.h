@@ -179,7 +179,7 @@ DG_API dg_status dg_project(const float* params, int64_t stride, int64_t P, cons
 DG_API size_t dg_bin_workspace_size(int64_t P, int32_t n_views, int64_t M_cap);
 
 /* Phase 1: orders the visible records by (view, depth bits, index) and
- * computes each one's first pair slot.  Writes the total pair count M to
+ * counts their pairs.  Writes the total pair count M to
  * *M_out (device int64).  The caller reads M (or checks it against its
  * capacity) before phase 2.  ws/ws_bytes: workspace from
  * dg_bin_workspace_size with the same P and n_views; its content carries
@@ -189,15 +189,17 @@ DG_API dg_status dg_bin_count(const float* depth, const int32_t* tiles, int64_t 
                        size_t ws_bytes, int64_t M_cap, int64_t* M_out, dg_stream stream);
 
 /* Phase 2: emits the pairs in (view, depth) order and stably sorts them by
- * global tile id.  A record whose feat holds a tile mask (opts->tight_bins
+ * global tile id.  The pair counts follow from feat and radius, and have to be
+ * those of phase 1's tiles.  A record whose feat holds a tile mask (opts->tight_bins
  * of dg_project) gets pairs only for the mask's tiles.
  * Out: gid    [M_cap] uint32, record index v * P + i of each sorted pair;
  *      ranges [2 * total tiles] uint32, [start, end) of each tile's list;
  *      status (device int32): 0, or DG_ERR_CAPACITY when M > M_cap, in which
  *              case gid is untouched and every range is empty, or
  *              DG_ERR_TIMEOUT when a bounded wait between thread blocks of
- *              phase 1 gave up (lists not valid; does not happen when the
- *              device runs the launch to completion).
+ *              gave up (lists not valid; does not happen when the device
+ *              runs the launch to completion), or DG_ERR_CUDA when the records'
+ *              pairs are not those counted in phase 1 (every range is empty).
  * feat/radius are dg_project's outputs for the same P and cameras. */
 DG_API dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64_t P, const dg_camera* cams,
                       int32_t n_views, int32_t tile, void* ws, size_t ws_bytes, int64_t M_cap, uint32_t* gid,

@@ -326,7 +326,7 @@ extern "C" dg_status dg_densify_apply(const float* params, const float* m, const
             dg::k_cand_keys<<<gb, 256, 0, s>>>(w.flags, w.score, w.cpos, (int)P, w.k0, w.v0);
             dg_note_launch();
             dg::SortBufs sb{w.hist, w.bsum};
-            const dg::KV r = dg::radix_sort(w.k0, w.v0, w.k1, w.v1, nullptr, nullptr, nullptr, n_cand, 32, sb, s);
+            const dg::KV r = dg::radix_sort(w.k0, w.v0, w.k1, w.v1, nullptr, n_cand, 32, sb, s);
             dg::k_mark_selected<<<(int)((n_sel + 255) / 256), 256, 0, s>>>(r.v, n_sel, w.flags);
             dg_note_launch();
         } else {

@@ -1,26 +1,40 @@
-// onesweep.cuh -- single-pass radix passes and a single-pass exclusive scan,
-// both built on decoupled look-back (Merrill & Garland, "Single-pass Parallel
+// onesweep.cuh -- stable single-kernel radix passes over the views of a batch,
+// built on decoupled look-back (Merrill & Garland, "Single-pass Parallel
 // Prefix Scan with Decoupled Look-back", 2016; the radix form follows
 // Adinets & Merrill, "Onesweep: A Faster Least Significant Digit Radix Sort
-// for GPUs", 2022).  Used by the binning stages, where the classic
-// histogram -> scan -> scatter passes spent most of their time in launch
-// gaps.
+// for GPUs", 2022).  Both stages of the binning use them: the depth order of
+// the records and the tile order of the pairs.
+//
+// Segments.  Each view's items are a segment of their own: a block belongs to
+// one view, counts and look-back stay within it, and the view index is never a
+// sort digit.  (Sorting all views as one sequence took one more pass over the
+// records and, at 16 views of 1237x822, three 6-bit passes over the pairs
+// instead of two 7-bit ones.)
 //
 // A pass is one kernel.  Each CTA takes a tile number from a counter when it
-// starts, ranks its RS_TILE keys by digit (warp match_any within warp-owned
-// segments, so the pass is stable), publishes its per-digit totals, and sums
-// the totals of the tiles before it by walking back over their published
-// words until one holds an inclusive prefix.  A CTA only waits on tiles taken
-// by CTAs that started before it and that never wait on a later tile, so every
-// wait ends; each is bounded all the same, and a wait that gives up records
-// DG_ERR_TIMEOUT and carries on with what it has.
+// starts, ranks its THREADS x IPT items by digit within warp-owned segments
+// (so the pass is stable), publishes its per-digit totals, and sums the totals
+// of its view's earlier tiles by walking back over their published words until
+// one holds an inclusive prefix.  A CTA only waits on tiles taken by CTAs that
+// started before it and that never wait on a later tile, so every wait ends;
+// each is bounded all the same, and a wait that gives up records
+// DG_ERR_TIMEOUT and carries on with what it has.  The start of each digit
+// comes from the digit counts of the whole view, counted before the first pass
+// and scanned by every CTA together with its own totals.
 //
-// The global start of each digit comes from the histograms of all passes,
-// counted in one read of the keys before the first pass (a one-CTA kernel
-// scans them).  Look-back words are cleared one pass ahead: the
-// histogram kernel clears the first pass's words, pass p clears the words of
-// pass p + 1 (the two alternate between two regions), so no pass needs a
-// separate clearing launch.
+// What bounds a pass: about 170 instructions per warp and 32 items at 40% of
+// the issue slots, the rest waits (a lone tile's chain of ticket, loads, ranking,
+// prefix, look-back and scatter takes 7-9 us), not its 16 B per item.  Measured
+// on 1.7M (key, value) items with 8-bit digits: 32 us with 2048-item tiles,
+// 64-bit words, a 16-word look-back window polled without pause and 64-bit
+// match masks; 22 us with 4096-item tiles, a 4-word window and a pause between
+// polls (more words in flight flood L2: a 32-word window took 55 us).  Four
+// votes' worth of instructions per digit bit became four instructions, and a
+// value is loaded only after its rank is known, so that four CTAs fit an SM (on
+// 33M pairs 1.16 against 1.23 ms for the whole binning with three; tiles of
+// 2048, 3072 or 5120 items 1.40, 1.23 and 1.37).  At 100k items a 1024-item tile
+// takes 6 us against 9 for 4096: the small tile is used while the items fill at
+// most two of them per SM.
 #pragma once
 
 #include "radix.cuh"
@@ -28,28 +42,27 @@
 namespace dg {
 namespace {
 
-constexpr int OS_MAXPASS = 6;
-constexpr uint64_t kLbAgg = 1ull << 62;   // word holds the tile's own total
-constexpr uint64_t kLbInc = 2ull << 62;   // word holds the inclusive prefix
+constexpr int OS_THREADS = 256;
+constexpr int OS_WARPS = OS_THREADS / 32;
+constexpr int OS_BINS = 256;              // 8-bit digits, one thread per digit
+constexpr int OS_IPT_BIG = 16;
+constexpr int OS_IPT_SMALL = 4;
+constexpr long long OS_SMALL_MAX = 152LL * 2 * OS_THREADS * OS_IPT_SMALL;
+constexpr uint64_t kLbAgg = 1ull << 62;   // 64-bit word holding the tile's own total
+constexpr uint64_t kLbInc = 2ull << 62;   // 64-bit word holding the inclusive prefix
 constexpr uint64_t kLbCount = (1ull << 62) - 1;
 constexpr int kLbPolls = 1 << 20;         // polls of one word before giving up
 
-// Per-call control block, zeroed by the caller before the histogram kernel.
-// The histogram CTAs add their counts into one of OS_HCOPIES copies (by CTA
-// index) so that thousands of CTAs do not queue on the same 256 words.
-constexpr int OS_HCOPIES = 16;
-struct OsCtl {
-    uint32_t ctr[OS_MAXPASS];              // tile counters of the passes (and of the scan)
-    int32_t err;                           // DG_ERR_TIMEOUT once a wait gave up
-    uint32_t hist[OS_MAXPASS][OS_HCOPIES][1 << RS_MAXBITS];
-    uint32_t base[OS_MAXPASS][1 << RS_MAXBITS];  // exclusive scan of the summed counts
+// Look-back words: the top two bits hold the state (0 not published, 1 own
+// total, 2 inclusive prefix), the rest the count.  32-bit words serve segments
+// below 2^30 items, 64-bit ones the rest.
+template <typename Word>
+struct LbWord {
+    static constexpr int kShift = 8 * (int)sizeof(Word) - 2;
+    static constexpr Word kCount = ((Word)1 << kShift) - 1;
+    static __device__ __forceinline__ Word agg(Word c) { return ((Word)1 << kShift) | c; }
+    static __device__ __forceinline__ Word inc(Word c) { return ((Word)2 << kShift) | c; }
 };
-
-// This CTA's copy of pass p's counts.
-__device__ __forceinline__ uint32_t* os_hist(OsCtl* ctl, int p)
-{
-    return ctl->hist[p][blockIdx.x % OS_HCOPIES];
-}
 
 __device__ __forceinline__ uint64_t ld_relaxed(const uint64_t* p)
 {
@@ -57,38 +70,46 @@ __device__ __forceinline__ uint64_t ld_relaxed(const uint64_t* p)
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ void st_relaxed(uint64_t* p, uint64_t v)
 {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v)
+{
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 
 // Sum of the counts the tiles before tile t published in column d of a
-// [tiles][stride] word array, up to and including the nearest inclusive
-// word.  The words of OS_WINDOW predecessors are read at once: when every
-// tile publishes at about the same time, the walk back to an inclusive word
-// takes about sqrt(2 t / OS_WINDOW) round trips instead of sqrt(2 t).
-constexpr int OS_WINDOW = 16;
-__device__ inline uint64_t os_lookback(const uint64_t* look, long long t, int stride, int d, int* err,
-                                       int max_polls = kLbPolls)
+// [tiles][stride] word array, up to and including the nearest inclusive word;
+// OS_WINDOW predecessors are read at once.
+constexpr int OS_WINDOW = 4;
+template <typename Word>
+__device__ inline Word os_lookback(const Word* look, long long t, int stride, int d, int* err,
+                                   int max_polls = kLbPolls)
 {
-    uint64_t sum = 0;
+    Word sum = 0;
     long long j = t;  // the window covers tiles j - OS_WINDOW .. j - 1
     int polls = 0;
     while (j > 0) {
-        uint64_t w[OS_WINDOW];
+        Word w[OS_WINDOW];
 #pragma unroll
         for (int q = 0; q < OS_WINDOW; ++q)
-            w[q] = j - 1 - q >= 0 ? ld_relaxed(look + (j - 1 - q) * stride + d) : kLbInc;
+            w[q] = j - 1 - q >= 0 ? ld_relaxed(look + (j - 1 - q) * stride + d) : LbWord<Word>::inc(0);
         int used = OS_WINDOW;
 #pragma unroll
         for (int q = 0; q < OS_WINDOW; ++q) {
             if (used < OS_WINDOW) break;
-            const uint64_t st = w[q] >> 62;
+            const Word st = w[q] >> LbWord<Word>::kShift;
             if (st == 0) {
                 used = q;  // tile j - 1 - q has not published yet: read again from there
             } else {
-                sum += w[q] & kLbCount;
+                sum += w[q] & LbWord<Word>::kCount;
                 if (st == 2) return sum;
             }
         }
@@ -98,194 +119,341 @@ __device__ inline uint64_t os_lookback(const uint64_t* look, long long t, int st
                 atomicExch(err, DG_ERR_TIMEOUT);
                 return sum;
             }
-            __nanosleep(32);
+            __nanosleep(40);
         }
     }
     return sum;
 }
 
-// One CTA of 256 threads, launched after the histogram kernel: sums the
-// copies and writes the exclusive scan of each pass's counts to ctl->base.
-// (A separate launch instead of a last-CTA step: that step needs a fence
-// that makes every histogram CTA wait for its own output writes.)
-__global__ void __launch_bounds__(256) k_os_base(OsCtl* ctl, int npass)
+// The same sum for one column of 64-bit words, taken by a whole warp, 32
+// predecessors a time; false when a wait gave up.
+__device__ inline bool os_lookback_warp(const uint64_t* look, long long t, uint64_t* out, int lane)
 {
-    __shared__ uint32_t sm[33];
-    for (int p = 0; p < npass; ++p) {
-        uint32_t c = 0;
+    uint64_t& sum = *out;
+    sum = 0;
+    long long j = t;
+    int polls = 0;
+    while (j > 0) {
+        const uint64_t w = j - 1 - lane >= 0 ? ld_relaxed(look + (j - 1 - lane)) : kLbInc;
+        const uint32_t none = __ballot_sync(0xffffffffu, (w >> 62) == 0);
+        const uint32_t inc = __ballot_sync(0xffffffffu, (w >> 62) == 2);
+        // lanes before the first unpublished word and up to the first inclusive one
+        const int lim = none ? __ffs(none) - 1 : 32;
+        const int first = inc ? __ffs(inc) - 1 : 32;
+        const int use = first < lim ? first + 1 : lim;
+        uint64_t x = lane < use ? w & kLbCount : 0;
 #pragma unroll
-        for (int q = 0; q < OS_HCOPIES; ++q) c += ctl->hist[p][q][threadIdx.x];
-        uint32_t tot;
-        const uint32_t ex = block_excl_scan<uint32_t>(c, sm, &tot);
-        ctl->base[p][threadIdx.x] = ex;
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        sum += x;
+        if (first < lim) return true;
+        j -= use;
+        if (use < 32) {
+            if (++polls > kLbPolls) return false;
+            __nanosleep(40);
+        }
+    }
+    return true;
+}
+
+// The views' items: view v holds cnt[v] items (or `fixed` when cnt is null),
+// starting at v * stride, or right behind view v - 1's when stride < 0.  When
+// all views hold more than `cap` items together, or *bad is set, there is
+// nothing to do.
+struct Segs {
+    int V;
+    const unsigned long long* cnt;
+    long long fixed, stride, cap;
+    const int* bad;
+};
+
+// A block's tile: view (-1: none left), tile number in the view, the view's
+// item count, first item and first tile (over all views).
+struct SegTile {
+    int v;
+    uint32_t t;
+    long long n, off, tbase;
+};
+
+// Tile b of the views in `tile`-item tiles; called by one whole warp.
+__device__ inline void seg_tile(const Segs& sg, uint32_t b, int tile, SegTile* out, int lane)
+{
+    const long long n = lane < sg.V ? (sg.cnt ? (long long)sg.cnt[lane] : sg.fixed) : 0;
+    const long long nt = (n + tile - 1) / tile;
+    const long long nt_inc = warp_incl_scan<long long>(nt, lane);
+    const long long n_inc = warp_incl_scan<long long>(n, lane);
+    const long long total = __shfl_sync(0xffffffffu, n_inc, 31);
+    const bool run = total <= sg.cap && !(sg.bad && *sg.bad != 0);
+    const bool mine = run && lane < sg.V && (long long)b >= nt_inc - nt && (long long)b < nt_inc;
+    if (lane == 0) out->v = -1;
+    __syncwarp();
+    if (mine) {
+        out->v = lane;
+        out->t = (uint32_t)((long long)b - (nt_inc - nt));
+        out->n = n;
+        out->off = sg.stride < 0 ? n_inc - n : lane * sg.stride;
+        out->tbase = nt_inc - nt;
     }
 }
 
 struct OsPass {
-    uint64_t* look;        // [tiles][mask + 1] look-back words of this pass
-    uint64_t* look_next;   // the next pass's words, cleared here (null after the last pass)
-    int next_nbins;        // digits of the next pass
-    uint32_t* ctr;         // this pass's tile counter (zero before the launch)
-    const uint32_t* base;  // global start of each digit
+    void* look;            // [tiles][mask + 1] look-back words of this pass, zero before the launch
+    uint32_t* ctr;         // this pass's tile counter, zero before the launch
+    const uint32_t* hist;  // view v's digit counts of this pass at hist + v * hist_stride
+    int hist_stride;
+    uint32_t* hist_next;   // nullable: counts of the next digit to add this tile's to
+    uint32_t mask_next;
     int* err;
     int shift;
     uint32_t mask;
+    uint32_t* kout;        // nullable: values only
+    uint32_t* vout;
+    uint2* ranges;         // nullable: the last tile pass's ranges (complement of the start, end), zero before the launch
+    int xbits;             // with ranges: a key is tile row << xbits | tile column
+    int TX[DG_MAX_VIEWS], toff[DG_MAX_VIEWS + 1];  // with ranges: tiles per row and first tile of each view
+    const unsigned long long* m_views;  // nullable: the views' pair counts, summed into *m_ws and *m_out
+    long long* m_ws;
+    long long* m_out;
 };
 
-// Key sources of a pass: item i of the input gives (key, value).
+// Key sources of a pass: load() fills the warp-striped keys (item k of lane l
+// of warp w at position w * 32 IPT + 32 k + l of the tile) and returns the bit
+// mask of those that exist; values() fills their values, after the ranks are
+// known (held from the start they would not fit the registers of four CTAs per
+// SM).  sk, sv: IPT * OS_THREADS words of scratch each; sv is left as load()
+// wrote it until values() returns on every thread.
 struct SrcKV {
     const uint32_t* k;
     const uint32_t* v;
-    __device__ void operator()(long long i, uint32_t& key, uint32_t& val) const { key = k[i]; val = v[i]; }
+    template <int IPT>
+    __device__ __forceinline__ uint32_t load(const SegTile& st, int nv, uint32_t*, uint32_t*, uint32_t (&key)[IPT],
+                                             int warp, int lane) const
+    {
+        const int seg = warp * 32 * IPT + lane;
+        const uint32_t* kp = k + st.off + (long long)st.t * (OS_THREADS * IPT) + seg;
+        if (nv == OS_THREADS * IPT) {
+#pragma unroll
+            for (int i = 0; i < IPT; ++i) key[i] = kp[32 * i];
+            return (1u << IPT) - 1u;
+        }
+        uint32_t ok = 0;
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) {
+            const bool on = seg + 32 * i < nv;
+            key[i] = on ? kp[32 * i] : 0u;
+            ok |= (on ? 1u : 0u) << i;
+        }
+        return ok;
+    }
+    template <int IPT>
+    __device__ __forceinline__ void values(const SegTile& st, int nv, const uint32_t*, uint32_t (&val)[IPT], int warp,
+                                           int lane) const
+    {
+        const int seg = warp * 32 * IPT + lane;
+        const uint32_t* vp = v + st.off + (long long)st.t * (OS_THREADS * IPT) + seg;
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) val[i] = seg + 32 * i < nv ? vp[32 * i] : 0u;
+    }
 };
 
-// One stable pass on digit (key >> shift) & mask; kout may be null (values only).
-template <class Src>
-__global__ void __launch_bounds__(RS_THREADS, 4)
-k_os_pass(Src src, uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, const long long* n_dev,
-          long long n_cap, OsPass ps)
+// Lanes of the warp with this lane's NB-bit digit, among those in `on` (which
+// holds this lane): per digit bit one vote, and the vote or its complement kept
+// by the lane's own bit.
+template <int NB>
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d, uint32_t on)
 {
-    __shared__ uint32_t cnt[RS_WARPS][1 << RS_MAXBITS];
-    __shared__ uint32_t dstart[1 << RS_MAXBITS];
-    __shared__ uint32_t gstart[1 << RS_MAXBITS];
-    __shared__ uint32_t sk[RS_TILE];
-    __shared__ uint32_t sv[RS_TILE];
-    __shared__ uint32_t scan_sm[33];
-    __shared__ uint32_t s_t;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long n = eff_count(n_dev, n_cap);
-    if (threadIdx.x == 0) s_t = atomicAdd(ps.ctr, 1u);
-    __syncthreads();
-    const long long t = s_t;
-    const long long base = t * RS_TILE;
-    if (base >= n) return;
-    const int nbins = (int)ps.mask + 1;
-    if (ps.look_next)
-        for (int d = threadIdx.x; d < ps.next_nbins; d += RS_THREADS) ps.look_next[t * ps.next_nbins + d] = 0;
-    const long long seg = base + (long long)warp * (32 * RS_IPT);
-    for (int d = lane; d < nbins; d += 32) cnt[warp][d] = 0;
-    __syncwarp();
-    uint32_t key[RS_IPT], val[RS_IPT], rank[RS_IPT];
+    uint32_t m = on;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        asm("{\n\t.reg .pred p;\n\t.reg .b32 t, b;\n\t"
+            "and.b32 t, %1, %2;\n\t"
+            "setp.ne.u32 p, t, 0;\n\t"
+            "vote.sync.ballot.b32 b, p, 0xffffffff;\n\t"
+            "@p and.b32 %0, %0, b;\n\t"
+            "@!p lop3.b32 %0, %0, b, 0, 0x30;\n\t}"
+            : "+r"(m) : "r"(d), "r"(1u << q));
+    }
+    return m;
+}
+
+// Stable rank of a warp's items among its items of the same digit, in position
+// order; wcnt: the warp's running count per digit (zero on entry, the totals on
+// return).  FULL: every item exists.  NB: digit bits to vote on, 0 for
+// __match_any_sync (fewer instructions when a warp holds few distinct digits).
+template <int IPT, int NB, bool FULL>
+__device__ __forceinline__ void os_rank(const uint32_t (&key)[IPT], uint32_t (&rank)[IPT], uint32_t ok,
+                                        uint32_t shift, uint32_t mask, uint32_t* wcnt, int lane)
+{
     const uint32_t lt = (1u << lane) - 1u;
+    // all peer masks first, then the running counts (a chain through shared memory)
 #pragma unroll
-    for (int k = 0; k < RS_IPT; ++k) {
-        const long long i = seg + (long long)k * 32 + lane;
-        key[k] = 0u;
-        val[k] = 0u;
-        if (i < n) src(i, key[k], val[k]);
+    for (int k = 0; k < IPT; ++k) {
+        const uint32_t d = (key[k] >> shift) & mask;
+        const bool on = FULL || ((ok >> k) & 1u);
+        if (NB == 0) rank[k] = __match_any_sync(0xffffffffu, on ? d : 0x10000u + (uint32_t)lane);
+        else rank[k] = digit_peers<NB>(d, FULL ? 0xffffffffu : __ballot_sync(0xffffffffu, on));
     }
-    warp_rank(key, rank, seg, n, ps.shift, ps.mask, false, cnt[warp], lane, lt);
-    __syncthreads();
-    // per digit: exclusive prefix over warps (tile-local) and the tile total;
-    // the aggregate is published at once so that later tiles can pass it
-    uint32_t total = 0;
-    if ((int)threadIdx.x < nbins) {
-        const int d = threadIdx.x;
 #pragma unroll
-        for (int w = 0; w < RS_WARPS; ++w) {
-            const uint32_t c = cnt[w][d];
-            cnt[w][d] = total;
-            total += c;
+    for (int k = 0; k < IPT; ++k) {
+        const uint32_t m = rank[k];
+        uint32_t* c = wcnt + ((key[k] >> shift) & mask);
+        const uint32_t before = *c, below = __popc(m & lt);
+        __syncwarp();
+        if (below == 0 && (FULL || ((ok >> k) & 1u))) *c = before + __popc(m);
+        __syncwarp();
+        rank[k] = before + below;
+    }
+}
+
+// One stable pass on digit (key >> shift) & mask; NB as os_rank's (at least the
+// digit's width, or 0).
+template <int IPT, typename Word, int NB, class Src>
+__global__ void __launch_bounds__(OS_THREADS, IPT == OS_IPT_BIG ? 4 : 5)
+k_os_pass(Src src, Segs sg, OsPass ps)
+{
+    constexpr int TILE = OS_THREADS * IPT;
+    __shared__ uint32_t cnt[OS_WARPS][OS_BINS];  // per warp: items of a digit so far, then the digit's place in the tile
+    __shared__ uint32_t gstart[OS_BINS];
+    __shared__ __align__(16) uint32_t sk[TILE];
+    __shared__ __align__(16) uint32_t sv[TILE];
+    __shared__ uint64_t ssum[OS_WARPS];
+    __shared__ uint32_t hnext[OS_BINS];
+    __shared__ SegTile s_st;
+    __shared__ int s_bad;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    hnext[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_bad = 0;
+    if (warp == 0) {
+        uint32_t b = 0;
+        if (lane == 0) b = atomicAdd(ps.ctr, 1u);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        seg_tile(sg, b, TILE, &s_st, lane);
+        if (ps.m_views && b == 0 && lane == 0) {
+            unsigned long long m = 0;
+            for (int v = 0; v < sg.V; ++v) m += ps.m_views[v];
+            *ps.m_ws = (long long)m;
+            *ps.m_out = (long long)m;
         }
-        st_relaxed(ps.look + t * nbins + d, (t == 0 ? kLbInc : kLbAgg) | total);
     }
-    uint32_t all;
-    const uint32_t ex = block_excl_scan<uint32_t>(total, scan_sm, &all);
-    if ((int)threadIdx.x < nbins) dstart[threadIdx.x] = ex;
+    const int nbins = (int)ps.mask + 1;
+    const int d0 = threadIdx.x;
+    uint32_t* wcnt = cnt[warp];
+    for (int d = lane; d < nbins; d += 32) wcnt[d] = 0;
     __syncthreads();
-    // stage the tile in digit order (the keys' registers are free after this)
+    const SegTile& st = s_st;
+    if (st.v < 0) return;
+    const uint32_t hv = d0 < nbins ? ps.hist[(long long)st.v * ps.hist_stride + d0] : 0u;
+    Word* look = (Word*)ps.look + (st.tbase + st.t) * nbins;  // this tile's words; earlier tiles' before them
+    const long long rest = st.n - (long long)st.t * TILE;
+    const int nv = rest < TILE ? (int)rest : TILE;
+    const uint32_t shift = (uint32_t)ps.shift, mask = ps.mask;
+    uint32_t key[IPT], rank[IPT];
+    const uint32_t ok = src.template load<IPT>(st, nv, sk, sv, key, warp, lane);
+    const bool full = __all_sync(0xffffffffu, ok == (1u << IPT) - 1u);
+    if (full) os_rank<IPT, NB, true>(key, rank, ok, shift, mask, wcnt, lane);
+    else os_rank<IPT, NB, false>(key, rank, ok, shift, mask, wcnt, lane);
+    if (ps.hist_next) {
+        const int sh = ps.shift + __popc(mask);
+        const uint32_t mn = ps.mask_next;
 #pragma unroll
-    for (int k = 0; k < RS_IPT; ++k) {
-        const long long i = seg + (long long)k * 32 + lane;
-        if (i < n) {
-            const uint32_t d = (key[k] >> ps.shift) & ps.mask;
-            const uint32_t p = dstart[d] + cnt[warp][d] + rank[k];
+        for (int k = 0; k < IPT; ++k)
+            if (full || ((ok >> k) & 1u)) atomicAdd(&hnext[(key[k] >> sh) & mn], 1u);
+    }
+    __syncthreads();
+    // per digit the tile's total, published at once so that later tiles can pass it
+    uint32_t total = 0;
+    if (d0 < nbins) {
+#pragma unroll
+        for (int w = 0; w < OS_WARPS; ++w) total += cnt[w][d0];
+        st_relaxed(look + d0, st.t == 0 ? LbWord<Word>::inc(total) : LbWord<Word>::agg(total));
+    }
+    // one scan for the tile's digit starts (low half) and the view's (high half)
+    const uint64_t both = (uint64_t)total | ((uint64_t)hv << 32);
+    const uint64_t inc = warp_incl_scan<uint64_t>(both, lane);
+    if (lane == 31) ssum[warp] = inc;
+    __syncthreads();
+    uint64_t ex = inc - both;
+    uint32_t have = 0;
+#pragma unroll
+    for (int w = 0; w < OS_WARPS; ++w) {
+        const uint64_t x = ssum[w];
+        ex += w < warp ? x : 0;
+        have += (uint32_t)x;
+    }
+    if (d0 < nbins) {
+        uint32_t run = (uint32_t)ex;
+#pragma unroll
+        for (int w = 0; w < OS_WARPS; ++w) {
+            const uint32_t c = cnt[w][d0];
+            cnt[w][d0] = run;
+            run += c;
+        }
+    }
+    if (ps.hist_next && threadIdx.x <= ps.mask_next && hnext[threadIdx.x])
+        atomicAdd(&ps.hist_next[(long long)st.v * ps.hist_stride + threadIdx.x], hnext[threadIdx.x]);
+    uint32_t val[IPT];
+    src.template values<IPT>(st, nv, sv, val, warp, lane);
+    __syncthreads();
+    // stage the tile in digit order
+#pragma unroll
+    for (int k = 0; k < IPT; ++k) {
+        if (full || ((ok >> k) & 1u)) {
+            const uint32_t p = wcnt[(key[k] >> shift) & mask] + rank[k];
             sk[p] = key[k];
             sv[p] = val[k];
         }
     }
-    // global start of each digit: counts of all earlier tiles
-    if ((int)threadIdx.x < nbins) {
-        const int d = threadIdx.x;
+    // the digit's place among the view's items: its start, plus the counts of earlier tiles
+    if (d0 < nbins) {
         uint32_t before = 0;
-        if (t > 0) {
-            before = (uint32_t)os_lookback(ps.look, t, nbins, d, ps.err);
-            st_relaxed(ps.look + t * nbins + d, kLbInc | (uint64_t)(before + total));
+        if (st.t > 0) {
+            before = (uint32_t)os_lookback(look - (long long)st.t * nbins, st.t, nbins, d0, ps.err);
+            st_relaxed(look + d0, LbWord<Word>::inc((Word)before + (Word)total));
         }
-        gstart[d] = ps.base[d] + before;
+        const uint32_t at = (uint32_t)(ex >> 32) + before;
+        // (always inside the view's items, unless a wait gave up in this pass or before)
+        if ((unsigned long long)at + total > (unsigned long long)st.n) s_bad = 1;
+        gstart[d0] = (uint32_t)st.off + at - (uint32_t)ex;
     }
     __syncthreads();
-    const int nvalid = (int)((n - base) < RS_TILE ? (n - base) : RS_TILE);
-    for (int j = threadIdx.x; j < nvalid; j += RS_THREADS) {
-        const uint32_t kk = sk[j];
-        const uint32_t d = (kk >> ps.shift) & ps.mask;
-        const uint32_t pos = gstart[d] + (uint32_t)j - dstart[d];
-        if (kout) kout[pos] = kk;
-        vout[pos] = sv[j];
-    }
-}
-
-// Exclusive scan of ld(0..n) into out in one pass over SCAN_TILE-item tiles;
-// *total receives the sum.  look: one word per tile, zero before the launch;
-// ctr: zero before the launch.
-template <typename Load>
-__global__ void __launch_bounds__(SCAN_THREADS)
-k_os_scan(Load ld, long long n, uint64_t* __restrict__ out, uint64_t* look, uint32_t* ctr, long long* total,
-          int* err)
-{
-    // one pad word per 16 keeps both the coalesced and the per-thread accesses
-    // free of bank conflicts
-    __shared__ uint64_t s_buf[SCAN_TILE + SCAN_TILE / 16];
-    auto at = [](int i) { return i + (i >> 4); };
-    __shared__ uint64_t sm[33];
-    __shared__ uint32_t s_t;
-    __shared__ uint64_t s_ex;
-    if (threadIdx.x == 0) s_t = atomicAdd(ctr, 1u);
-    __syncthreads();
-    const long long t = s_t;
-    const long long ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-    if (t >= ntiles) return;
-    const long long tb = t * SCAN_TILE;
-    // coalesced load, then each thread takes SCAN_IPT consecutive items
+    if (s_bad) return;
+    uint32_t* const vout = ps.vout;
+    uint32_t* const kout = ps.kout;
+    if (kout) {
 #pragma unroll
-    for (int k = 0; k < SCAN_IPT; ++k) {
-        const long long i = tb + (long long)k * SCAN_THREADS + threadIdx.x;
-        s_buf[at(k * SCAN_THREADS + threadIdx.x)] = i < n ? ld(i) : 0;
-    }
-    __syncthreads();
-    uint64_t v[SCAN_IPT];
-    uint64_t acc = 0;
-#pragma unroll
-    for (int k = 0; k < SCAN_IPT; ++k) {
-        v[k] = s_buf[at(threadIdx.x * SCAN_IPT + k)];
-        acc += v[k];
-    }
-    uint64_t tot;
-    uint64_t run = block_excl_scan<uint64_t>(acc, sm, &tot);  // ends with a barrier
-    // in-tile exclusive prefixes first (frees v before the look-back)
-#pragma unroll
-    for (int k = 0; k < SCAN_IPT; ++k) {
-        s_buf[at(threadIdx.x * SCAN_IPT + k)] = run;
-        run += v[k];
-    }
-    if (threadIdx.x == 0) {
-        uint64_t ex = 0;
-        if (t == 0) {
-            st_relaxed(look, kLbInc | tot);
-        } else {
-            st_relaxed(look + t, kLbAgg | tot);
-            ex = os_lookback(look, t, 1, 0, err);
-            st_relaxed(look + t, kLbInc | ((ex + tot) & kLbCount));
+        for (int k = 0; k < IPT; ++k) {
+            const uint32_t j = threadIdx.x + k * OS_THREADS;
+            if (j >= have) break;
+            const uint32_t kk = sk[j], pos = gstart[(kk >> shift) & mask] + j;
+            kout[pos] = kk;
+            vout[pos] = sv[j];
         }
-        s_ex = ex;
-        if (t == ntiles - 1) *total = (long long)(ex + tot);
-    }
-    __syncthreads();
-    const uint64_t ex = s_ex;
+    } else {
 #pragma unroll
-    for (int k = 0; k < SCAN_IPT; ++k) {
-        const long long i = tb + (long long)k * SCAN_THREADS + threadIdx.x;
-        if (i < n) out[i] = ex + s_buf[at(k * SCAN_THREADS + threadIdx.x)];
+        for (int k = 0; k < IPT; ++k) {
+            const uint32_t j = threadIdx.x + k * OS_THREADS;
+            if (j >= have) break;
+            vout[gstart[(sk[j] >> shift) & mask] + j] = sv[j];
+        }
+    }
+    if (ps.ranges && total > 0) {
+        // the staged tile is in full key order (earlier passes sorted the lower
+        // bits), so each key is one run of it whose ends extend the key's range;
+        // mostly the tile holds one value of the lower bits: one key per digit
+        const uint32_t TX = (uint32_t)ps.TX[st.v], nt = (uint32_t)(ps.toff[st.v + 1] - ps.toff[st.v]);
+        uint2* const rg = ps.ranges + ps.toff[st.v];
+        const uint32_t g = gstart[d0], j1 = (uint32_t)ex + total;
+        for (uint32_t j = (uint32_t)ex; j < j1;) {
+            const uint32_t kk = sk[j];
+            uint32_t e = j1;
+            if (sk[j1 - 1] != kk)
+                for (e = j + 1; sk[e] == kk; ++e) {}
+            const uint32_t tile = (kk >> ps.xbits) * TX + (kk & ((1u << ps.xbits) - 1u));
+            if (tile < nt) {
+                atomicMax(&rg[tile].x, ~(g + j));
+                atomicMax(&rg[tile].y, g + e);
+            }
+            j = e;
+        }
     }
 }
 

@@ -1,13 +1,13 @@
-// radix.cuh -- device-wide exclusive scan and stable LSD radix sort of
-// (uint32 key, uint32 value) pairs, shared by the binning and densification
-// kernels.  Kernels live in an anonymous namespace: each including
-// translation unit gets its own copy.
+// radix.cuh -- device-wide exclusive scan (densification, render split plan) and
+// stable LSD radix sort of (uint32 key, uint32 value) pairs (densification).
+// Kernels live in an anonymous namespace: each including translation unit gets
+// its own copy.
 //
 // Radix pass = per-block digit histogram, exclusive scan of the digit-major
 // histogram, stable scatter.  Each warp owns a contiguous segment of a block's
-// tile and finds the lanes with equal digits by one ballot per digit bit;
-// per-warp digit counts give the block-local offsets, so the scatter is
-// stable without a block-wide sort.
+// tile and finds the lanes with equal digits by __match_any_sync; per-warp digit
+// counts give the block-local offsets, so the scatter is stable without a
+// block-wide sort.
 #pragma once
 
 #include "common.cuh"
@@ -25,47 +25,19 @@ constexpr int RS_IPT = 8;
 constexpr int RS_TILE = RS_THREADS * RS_IPT;
 constexpr int RS_MAXBITS = 8;
 
-// Lanes of the warp holding the same `nbits`-bit digit as this lane, among the
-// lanes with ok set (the mask __match_any_sync would give over those lanes),
-// from one ballot per digit bit: the cost does not grow with the number of
-// distinct digits in the warp.  A lane without ok gets its own bit only.
-__device__ __forceinline__ uint32_t warp_peers(uint32_t d, int nbits, bool ok, int lane)
-{
-    uint32_t m = __ballot_sync(0xffffffffu, ok);
-#pragma unroll
-    for (int b = 0; b < RS_MAXBITS; ++b) {
-        if (b < nbits) {
-            const bool bit = (d >> b) & 1u;
-            const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-            m &= bit ? bal : ~bal;
-        }
-    }
-    return ok ? m : (1u << lane);
-}
-
 // Stable rank of a warp's RS_IPT x 32 keys (item k of lane l at position
 // seg + 32 k + l, valid below n) among the equal digits of the warp's
 // segment, in position order; wcnt: the warp's running count of each digit
-// (zero on entry, the digit totals on return).  Peer masks by ballots
-// (`ballot`: fixed cost, for digits that are nearly all distinct within a
-// warp) or by __match_any_sync (fast when a warp holds few distinct digits).
+// (zero on entry, the digit totals on return).
 __device__ __forceinline__ void warp_rank(const uint32_t (&key)[RS_IPT], uint32_t (&rank)[RS_IPT], long long seg,
-                                          long long n, int shift, uint32_t mask, bool ballot, uint32_t* wcnt,
-                                          int lane, uint32_t lt)
+                                          long long n, int shift, uint32_t mask, uint32_t* wcnt, int lane, uint32_t lt)
 {
-    const int nbits = __popc(mask);
     uint32_t peers[RS_IPT];
-    if (ballot) {
 #pragma unroll
-        for (int k = 0; k < RS_IPT; ++k)
-            peers[k] = warp_peers((key[k] >> shift) & mask, nbits, seg + (long long)k * 32 + lane < n, lane);
-    } else {
-#pragma unroll
-        for (int k = 0; k < RS_IPT; ++k) {
-            // out-of-range lanes get a digit no valid lane can have
-            const bool ok = seg + (long long)k * 32 + lane < n;
-            peers[k] = __match_any_sync(0xffffffffu, ok ? ((key[k] >> shift) & mask) : (0x10000u + (uint32_t)lane));
-        }
+    for (int k = 0; k < RS_IPT; ++k) {
+        // out-of-range lanes get a digit no valid lane can have
+        const bool ok = seg + (long long)k * 32 + lane < n;
+        peers[k] = __match_any_sync(0xffffffffu, ok ? ((key[k] >> shift) & mask) : (0x10000u + (uint32_t)lane));
     }
 #pragma unroll
     for (int k = 0; k < RS_IPT; ++k) {
@@ -117,12 +89,6 @@ struct LoadU32 {
     const uint32_t* a;
     __device__ uint64_t operator()(long long i) const { return a[i]; }
 };
-struct LoadTilesInOrder {  // tiles touched by the Gaussian at sorted position s
-    const int* tiles;
-    const uint32_t* order;
-    __device__ uint64_t operator()(long long s) const { return (uint64_t)tiles[order[s]]; }
-};
-
 template <typename Load>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(Load ld, long long n, uint64_t* bsum)
 {
@@ -222,14 +188,13 @@ k_rs_hist(const uint32_t* __restrict__ keys, const long long* n_dev, long long n
 }
 
 // Stable scatter of one radix pass.  Ranks are computed per warp-owned
-// segment (ballot peer masks within each 32-item round, running per-warp digit
-// counts), the block's items are first placed in shared memory in digit order,
+// segment (peer masks within each 32-item round, running per-warp digit counts), the block's items are first placed in shared memory in digit order,
 // then written out so that consecutive threads write consecutive addresses of
 // each digit's run.  kout may be null (values only).
 __global__ void __launch_bounds__(RS_THREADS, 4)
 k_rs_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
              uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, const long long* n_dev,
-             long long n_cap, int shift, uint32_t mask, bool ballot, const uint32_t* __restrict__ offs, int nblk)
+             long long n_cap, int shift, uint32_t mask, const uint32_t* __restrict__ offs, int nblk)
 {
     __shared__ uint32_t cnt[RS_WARPS][1 << RS_MAXBITS];
     __shared__ uint32_t dstart[1 << RS_MAXBITS];
@@ -254,7 +219,7 @@ k_rs_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
         key[k] = i < n ? kin[i] : 0u;
         val[k] = i < n ? vin[i] : 0u;
     }
-    warp_rank(key, rank, seg, n, shift, mask, ballot, cnt[warp], lane, lt);
+    warp_rank(key, rank, seg, n, shift, mask, cnt[warp], lane, lt);
     __syncthreads();
     // per digit: exclusive prefix over warps (block-local), digit total, global start
     uint32_t total = 0;
@@ -298,25 +263,15 @@ struct SortBufs {
     uint64_t* bsum;   // scan block sums
 };
 
-// Stable LSD sort of (key, val) over the low `bits` key bits.  Input in
-// (k0, v0); (k1, v1) is ping-pong space.  The last pass writes to
-// (kfin, vfin) when vfin is given (kfin may then be null: values only; they
-// must not alias k0/k1, v0/v1), else to the ping-pong buffer whose turn it
-// is.  When hist0_ready, the caller already wrote pass 0's per-block
-// histogram into sb.hist.  Returns where the result lies.
+// Stable LSD sort of n (key, val) over the low `bits` key bits.  Input in
+// (k0, v0); (k1, v1) is ping-pong space.  Returns where the result lies.
 struct KV { uint32_t* k; uint32_t* v; };
 
-static KV radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t* kfin,
-                     uint32_t* vfin, const long long* n_dev, long long n_cap, int bits,
-                     const SortBufs& sb, cudaStream_t s, bool hist0_ready = false, uint32_t ballot_passes = 0)
+static KV radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, const long long* n_dev, long long n_cap,
+                     int bits, const SortBufs& sb, cudaStream_t s)
 {
     const int nblk = (int)((n_cap + RS_TILE - 1) / RS_TILE);
     if (nblk == 0) return KV{k0, v0};
-    if (bits == 0) {
-        if (kfin) cudaMemcpyAsync(kfin, k0, sizeof(uint32_t) * n_cap, cudaMemcpyDeviceToDevice, s);
-        if (vfin) cudaMemcpyAsync(vfin, v0, sizeof(uint32_t) * n_cap, cudaMemcpyDeviceToDevice, s);
-        return KV{kfin ? kfin : k0, vfin ? vfin : v0};
-    }
     const int npass = (bits + RS_MAXBITS - 1) / RS_MAXBITS;
     const int per = (bits + npass - 1) / npass;
     uint32_t *ks = k0, *vs = v0;
@@ -324,31 +279,18 @@ static KV radix_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uin
         const int shift = p * per;
         const int b = (bits - shift) < per ? (bits - shift) : per;
         const uint32_t mask = (1u << b) - 1u;
-        const bool last = p == npass - 1;
-        uint32_t* kd = (last && vfin) ? kfin : (ks == k0 ? k1 : k0);
-        uint32_t* vd = (last && vfin) ? vfin : (vs == v0 ? v1 : v0);
-        if (!(p == 0 && hist0_ready)) {
-            k_rs_hist<<<nblk, RS_THREADS, 0, s>>>(ks, n_dev, n_cap, shift, mask, sb.hist, nblk);
-            dg_note_launch();
-        }
+        uint32_t* kd = ks == k0 ? k1 : k0;
+        uint32_t* vd = vs == v0 ? v1 : v0;
+        k_rs_hist<<<nblk, RS_THREADS, 0, s>>>(ks, n_dev, n_cap, shift, mask, sb.hist, nblk);
+        dg_note_launch();
         const long long nh = (long long)(mask + 1) * nblk;
         exclusive_scan(LoadU32{sb.hist}, nh, sb.hist, sb.bsum, (long long*)nullptr, s);
-        k_rs_scatter<<<nblk, RS_THREADS, 0, s>>>(ks, vs, kd, vd, n_dev, n_cap, shift, mask, (ballot_passes >> p) & 1u,
-                                                 sb.hist, nblk);
+        k_rs_scatter<<<nblk, RS_THREADS, 0, s>>>(ks, vs, kd, vd, n_dev, n_cap, shift, mask, sb.hist, nblk);
         dg_note_launch();
         ks = kd;
         vs = vd;
     }
     return KV{ks, vs};
-}
-
-// Digit width of the first pass of radix_sort over `bits` bits.
-static int first_pass_bits(int bits)
-{
-    if (bits == 0) return 0;
-    const int npass = (bits + RS_MAXBITS - 1) / RS_MAXBITS;
-    const int per = (bits + npass - 1) / npass;
-    return bits < per ? bits : per;
 }
 
 }  // namespace

@@ -3,96 +3,34 @@
 // The per-tile lists must come out ordered by (tile, depth bits, Gaussian
 // index).  Instead of one radix sort over 64-bit (tile | depth) keys of all
 // M pairs (6 passes of 8 bits), the order is built in two cheaper stages:
-//   1. a stable 32-bit LSD radix sort of the P visible depths (ties keep the
-//      index order), then an exclusive scan of the tile counts in that order;
+//   1. a stable 32-bit LSD radix sort of the visible depths (ties keep the
+//      index order);
 //   2. pairs are emitted in depth order, then stably sorted by tile id alone
-//      (ceil(log2(tiles)) bits: 2 passes at 1237x822 / 16^2 = 4056 tiles).
+//      (ceil(log2(tiles)) bits: 2 passes at 1237x822 / 8^2 = 15965 tiles).
 // Stability of stage 2 preserves the depth order inside each tile, so the
 // result equals the lexicographic (tile, depth bits, index) order.
-// Several views: records are r = v * P + i; stage 1 adds one stable pass on
-// the view index after the depth passes (order (view, depth, index)) and the
-// tile ids are global, view_offset[v] + ty * TX_v + tx, so each view's tiles
-// form one contiguous block of the range table.  The pair payload is the
-// record index r.
+// Several views: records are r = v * P + i; each view's records and pairs are
+// a segment sorted on its own (onesweep.cuh), with tile ids local to the view;
+// view v's pairs follow view v - 1's, and its ranges start at its first tile
+// of the global range table.  The pair payload is the record index r.
 //
-// Stage 1 runs each radix pass as one kernel with decoupled look-back
-// (onesweep.cuh), the digit counts of all passes counted in one read before
-// the first pass, and the tile-count scan likewise in one kernel.  Stage 2
-// keeps the classic pass (per-block digit histogram, scan of the
-// digit-major histogram, stable scatter; the first histogram comes out of
-// the emission kernel): measured on 8.2M pairs, the emission kernel's extra
-// work for all-pass counts cost more than the launches it saved.
-// Both rank equal digits within warp-owned segments (__match_any_sync, or
-// per-bit ballots on the low tile digit), so every pass is stable.
+// Stage 1 (dg_bin_count): one kernel counts the digits of all four depth
+// passes, the visible records and the pairs of each view; the first pass then
+// drops the culled records, so the other three move only the visible ones.
+// Stage 2 (dg_bin_sort): one kernel walks the records in depth order, forms
+// each one's tile rect (16 bytes), scans their pair counts (look-back) and
+// counts the tile digits of all passes, a run of tiles at a time; the first
+// tile pass emits its pairs straight into its ranking, so unsorted pairs never
+// reach memory; the last one extends the ranges of the tiles whose runs it
+// stages, so sorted keys are never stored.
+// Measured (2M Gaussians, one 1237x822 view, 5.9M pairs / 653k Gaussians, 16
+// views of 1237x822 to 309x205, 33M pairs): 0.315 / 1.16 ms both stages, against
+// 0.41 / 1.88 ms with all views sorted as one sequence, culled records carried
+// along, the pairs emitted to memory and histogram, scan and scatter kernels per
+// tile pass.
 #include "onesweep.cuh"
 
 namespace dg {
-
-// Tile-sort passes that rank by per-bit ballots instead of __match_any_sync
-// (bit p: pass p).  The low tile digit (neighbouring tiles of one Gaussian's
-// rectangle) is nearly all distinct within a warp; measured at 2M Gaussians,
-// ballots there took the pair sort from 0.266 to 0.244 ms, ballots on the high
-// digit too 0.256 ms.  The depth passes stay on __match_any_sync: ballots made
-// them slower on every digit (0.201 ms with none, 0.229 on the two low digits,
-// 0.255 on all four).
-constexpr uint32_t kTileBallotPasses = 0x1;
-
-// --------------------------------------------------------------- binning
-// Depth-order key of record i: its depth bits when it touches a tile, else
-// all ones (culled records sort last); the value is the record index.
-struct SrcDepth {
-    const float* depth;
-    const int* tiles;
-    __device__ void operator()(long long i, uint32_t& key, uint32_t& val) const
-    {
-        key = tiles[i] > 0 ? __float_as_uint(depth[i]) : 0xffffffffu;
-        val = (uint32_t)i;
-    }
-};
-
-// View key of the record r = v * P + i at a sorted position: its view v, or
-// n_views for a culled record, so that every culled record (no pairs) ends up
-// behind all visible records of all views.  (Left between two views, runs of
-// culled records would fill k_emit's window of staged Gaussians.)
-struct SrcView {
-    const uint32_t* order;
-    const int* tiles;
-    uint32_t P, n_views;
-    __device__ void operator()(long long i, uint32_t& key, uint32_t& val) const
-    {
-        val = order[i];
-        key = tiles[val] > 0 ? val / P : n_views;
-    }
-};
-
-// Digit counts of the four depth passes (and of the view pass when vbits >
-// 0) in one read of the depths; clears the first pass's look-back words.
-__global__ void __launch_bounds__(RS_THREADS)
-k_os_hist_depth(const float* __restrict__ depth, const int* __restrict__ tiles, long long N, uint32_t P,
-                uint32_t n_views, int vbits, OsCtl* ctl, uint64_t* __restrict__ look0)
-{
-    __shared__ uint32_t h[5][1 << RS_MAXBITS];
-    const int npass = vbits > 0 ? 5 : 4;
-    for (int i = threadIdx.x; i < 5 * (1 << RS_MAXBITS); i += RS_THREADS) (&h[0][0])[i] = 0;
-    __syncthreads();
-    const long long stride = (long long)gridDim.x * RS_THREADS;
-    for (long long i = (long long)blockIdx.x * RS_THREADS + threadIdx.x; i < N; i += stride) {
-        const bool vis = tiles[i] > 0;
-        const uint32_t k = vis ? __float_as_uint(depth[i]) : 0xffffffffu;
-        atomicAdd(&h[0][k & 255u], 1u);
-        atomicAdd(&h[1][(k >> 8) & 255u], 1u);
-        atomicAdd(&h[2][(k >> 16) & 255u], 1u);
-        atomicAdd(&h[3][k >> 24], 1u);
-        if (vbits > 0) atomicAdd(&h[4][vis ? (uint32_t)i / P : n_views], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < npass * (1 << RS_MAXBITS); i += RS_THREADS) {
-        const uint32_t c = (&h[0][0])[i];
-        if (c) atomicAdd(&os_hist(ctl, i >> RS_MAXBITS)[i & ((1 << RS_MAXBITS) - 1)], c);
-    }
-    const long long nw = (N + RS_TILE - 1) / RS_TILE * (1 << RS_MAXBITS);
-    for (long long i = (long long)blockIdx.x * RS_THREADS + threadIdx.x; i < nw; i += stride) look0[i] = 0;
-}
 
 struct TileGrid {
     int n;
@@ -100,280 +38,517 @@ struct TileGrid {
     int off[DG_MAX_VIEWS + 1];  // first global tile id of each view
 };
 
-// First sorted position whose pair range holds each RS_TILE block's first pair.
-__global__ void k_block_starts(const uint64_t* __restrict__ poff, long long P, const long long* M_dev, long long M_cap,
-                               int* __restrict__ bstart)
+constexpr int BIN_MAXPASS = 6;  // digits of a tile's column and row (at most 30 + 1 bits together)
+
+// Zeroed at the start of each phase: phase 1's counters ...
+struct BinCtl1 {
+    uint32_t ctr[4];
+    int32_t err;                                // DG_ERR_TIMEOUT once a wait gave up
+    unsigned long long nvis[DG_MAX_VIEWS];      // visible records of each view
+    unsigned long long npair[DG_MAX_VIEWS];     // pairs of each view
+    uint32_t hist[DG_MAX_VIEWS][4][OS_BINS];    // depth digit counts
+};
+// ... and phase 2's.
+struct BinCtl2 {
+    uint32_t ctr[1 + BIN_MAXPASS];              // records, tile passes
+    int32_t err;                                // DG_ERR_TIMEOUT or DG_ERR_CUDA
+    int32_t bad;                                // the records' pairs are not usable: emit nothing
+    uint32_t hist[DG_MAX_VIEWS][BIN_MAXPASS][OS_BINS];  // tile digit counts
+};
+
+// --------------------------------------------------------------- depth order
+constexpr int DH_THREADS = 512;
+constexpr int DH_IPT = 8;
+
+// Digit counts of the four depth passes and the visible records and pairs of
+// each view (blockIdx.y) in one read of depths and tile counts.
+__global__ void __launch_bounds__(DH_THREADS)
+k_depth_hist(const float* __restrict__ depth, const int* __restrict__ tiles, long long P, BinCtl1* ctl)
 {
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long M = *M_dev;
-    if (s >= P || M > M_cap) return;
-    const long long a = (long long)poff[s];
-    const long long e = s + 1 < P ? (long long)poff[s + 1] : M;
-    if (e <= a) return;
-    for (long long b = (a + RS_TILE - 1) / RS_TILE; b * RS_TILE < e; ++b) bstart[b] = (int)s;
+    __shared__ uint32_t h[4][OS_BINS];
+    __shared__ unsigned long long s_pairs;
+    for (int i = threadIdx.x; i < 4 * OS_BINS; i += DH_THREADS) (&h[0][0])[i] = 0;
+    if (threadIdx.x == 0) s_pairs = 0;
+    __syncthreads();
+    const int v = blockIdx.y;
+    const float* d = depth + (size_t)v * P;
+    const int* tl = tiles + (size_t)v * P;
+    unsigned long long pairs = 0;
+    for (long long base = (long long)blockIdx.x * (DH_THREADS * DH_IPT); base < P;
+         base += (long long)gridDim.x * (DH_THREADS * DH_IPT)) {
+        int n[DH_IPT];
+        uint32_t k[DH_IPT];
+#pragma unroll
+        for (int q = 0; q < DH_IPT; ++q) {
+            const long long i = base + q * DH_THREADS + threadIdx.x;
+            n[q] = i < P ? tl[i] : 0;
+            k[q] = i < P ? __float_as_uint(d[i]) : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < DH_IPT; ++q) {
+            if (n[q] > 0) {
+                pairs += (unsigned long long)n[q];
+                atomicAdd(&h[0][k[q] & 255u], 1u);
+                atomicAdd(&h[1][(k[q] >> 8) & 255u], 1u);
+                atomicAdd(&h[2][(k[q] >> 16) & 255u], 1u);
+                atomicAdd(&h[3][k[q] >> 24], 1u);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+    if ((threadIdx.x & 31) == 0 && pairs) atomicAdd(&s_pairs, pairs);
+    __syncthreads();
+    uint32_t* g = &ctl->hist[v][0][0];
+    uint32_t vis = 0;
+    for (int i = threadIdx.x; i < 4 * OS_BINS; i += DH_THREADS) {
+        const uint32_t c = (&h[0][0])[i];
+        if (c) atomicAdd(&g[i], c);
+        if (i < OS_BINS) vis += c;
+    }
+    vis = __reduce_add_sync(0xffffffffu, vis);
+    if ((threadIdx.x & 31) == 0 && vis) atomicAdd(&ctl->nvis[v], (unsigned long long)vis);
+    if (threadIdx.x == 0 && s_pairs) atomicAdd(&ctl->npair[v], s_pairs);
 }
 
-// Pair emission, one RS_TILE block of consecutive pairs per CTA.  The block's
-// Gaussians (at most RS_TILE, all with >= 1 pair) are staged in shared memory
-// with their rects; each pair finds its Gaussian by binary search over the
-// staged starts.  Writes key = tile id and value = Gaussian index, coalesced,
-// and the per-block histogram of the first radix digit.
-__global__ void __launch_bounds__(RS_THREADS)
-k_emit(const float4* __restrict__ feat, const int* __restrict__ radius, const uint32_t* __restrict__ order,
-       const uint64_t* __restrict__ poff, const int* __restrict__ bstart, long long P, uint32_t Pv,
-       const long long* M_dev, long long M_cap, int B, TileGrid tg, uint32_t mask0, uint32_t* __restrict__ pkey,
-       uint32_t* __restrict__ pval, uint32_t* __restrict__ hist0, int nblk, const int* __restrict__ err1,
-       int* status)
+// First depth pass: the visible records of the view, key = depth bits.
+struct SrcDepth {
+    const float* depth;
+    const int* tiles;
+    template <int IPT>
+    __device__ __forceinline__ uint32_t load(const SegTile& st, int nv, uint32_t*, uint32_t*, uint32_t (&key)[IPT],
+                                             int warp, int lane) const
+    {
+        const int seg = warp * 32 * IPT + lane;
+        const long long first = st.off + (long long)st.t * (OS_THREADS * IPT) + seg;
+        const float* dp = depth + first;
+        const int* tp = tiles + first;
+        uint32_t ok = 0;
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) {
+            const bool on = seg + 32 * i < nv;
+            key[i] = on ? __float_as_uint(dp[32 * i]) : 0u;
+            ok |= (on && tp[32 * i] > 0 ? 1u : 0u) << i;
+        }
+        return ok;
+    }
+    template <int IPT>
+    __device__ __forceinline__ void values(const SegTile& st, int, const uint32_t*, uint32_t (&val)[IPT], int warp,
+                                           int lane) const
+    {
+        const uint32_t first = (uint32_t)(st.off + (long long)st.t * (OS_THREADS * IPT)) + warp * 32 * IPT + lane;
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) val[i] = first + 32 * i;
+    }
+};
+
+// --------------------------------------------------------------- records in depth order
+constexpr int REC_IPT = 4;
+constexpr int REC_TILE = OS_THREADS * REC_IPT;
+
+// Tile keys: tile row << xbits | tile column, so that the lowest digits are the
+// column's and a record's counts of them take one addition per column of its
+// mask (or two for a rect of any size, into a difference array).  Grids whose
+// keys fit one digit (at most 8 bits) are sorted by the whole key.
+struct TileKey {
+    int xbits, bits;
+    int npass;
+    int shift[BIN_MAXPASS], width[BIN_MAXPASS];  // digits
+};
+
+static TileKey tile_key(const TileGrid& tg)
 {
-    const uint32_t n_tiles = (uint32_t)tg.off[tg.n];
-    // staged Gaussians: pair offset relative to the block (the first one's,
-    // <= 0, in s_first; the others' lie in 1 .. RS_TILE - 1), rect corner,
-    // rect width and view, record index, tile mask (0: every tile of the rect)
-    __shared__ uint16_t w_start[RS_TILE];
-    __shared__ uint32_t w_xy[RS_TILE];    // rect x0 | y0 << 16
-    __shared__ uint32_t w_wv[RS_TILE];    // rect width in tiles | view << 16
-    __shared__ uint32_t w_g[RS_TILE];     // record index
-    __shared__ unsigned long long w_m[RS_TILE];
-    __shared__ int s_first;
-    __shared__ int s_off[DG_MAX_VIEWS];   // global tile id of each view's tile (0, 0)
-    __shared__ int s_tx[DG_MAX_VIEWS];    // tiles per row of each view
-    __shared__ uint32_t h[1 << RS_MAXBITS];
-    const long long M = *M_dev;
-    // a failed wait of the depth order (phase 1) is reported here
-    if (blockIdx.x == 0 && threadIdx.x == 0 && *err1 != 0) *status = *err1;
-    if (M > M_cap) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) *status = DG_ERR_CAPACITY;
-        return;
+    TileKey k{};
+    int yb = 0;
+    for (int v = 0; v < tg.n; ++v) {
+        while ((1ll << k.xbits) < tg.TX[v]) ++k.xbits;
+        while ((1ll << yb) < tg.TY[v]) ++yb;
     }
-    // (status was cleared by the host before this launch; blocks only set errors)
-    __shared__ int s_nw;
-    for (int d = threadIdx.x; d < (1 << RS_MAXBITS); d += RS_THREADS) h[d] = 0;
-    for (int v = threadIdx.x; v < tg.n; v += RS_THREADS) {
-        s_off[v] = tg.off[v];
-        s_tx[v] = tg.TX[v];
+    k.bits = k.xbits + yb;
+    if (k.bits <= 8) {
+        k.npass = 1;
+        k.width[0] = k.bits > 0 ? k.bits : 1;
+        return k;
     }
-    if (threadIdx.x == 0) s_nw = 0;
-    __syncthreads();
-    const long long base = (long long)blockIdx.x * RS_TILE;
-    if (base < M) {  // block-uniform
-        const long long end = (base + RS_TILE) < M ? (base + RS_TILE) : M;
-        const int s_lo = bstart[blockIdx.x];
-        // stage the Gaussians whose pair range starts before `end` (a prefix of
-        // s_lo, s_lo + 1, ...).  A candidate's pair offset and record index are
-        // loaded together (both follow from its sorted position), then its
-        // record; each link is issued for all of a thread's candidates at once,
-        // the second half of the candidates only when the block holds more
-        // than RS_TILE / 2 Gaussians (fewer than 4 pairs each).
-        constexpr int HALF = RS_IPT / 2;
-        long long st[RS_IPT];
-        uint32_t gk[RS_IPT];
-#pragma unroll
-        for (int k = 0; k < HALF; ++k) {
-            const long long s = (long long)s_lo + threadIdx.x + k * RS_THREADS;
-            st[k] = s < P ? (long long)poff[s] : LLONG_MAX;
-            gk[k] = s < P ? order[s] : 0u;
-        }
-        const bool more = __syncthreads_or(st[HALF - 1] < end) != 0;
-#pragma unroll
-        for (int k = HALF; k < RS_IPT; ++k) {
-            const long long s = (long long)s_lo + threadIdx.x + k * RS_THREADS;
-            st[k] = more && s < P ? (long long)poff[s] : LLONG_MAX;
-            gk[k] = more && s < P ? order[s] : 0u;
-        }
-        int top = 0;
-#pragma unroll
-        for (int k = 0; k < RS_IPT; ++k) {
-            if (st[k] < end) {
-                const int w = (int)threadIdx.x + k * RS_THREADS;
-                const uint32_t g = gk[k];
-                const int v = (int)(g / Pv);
-                const float4 f0 = feat[3 * (size_t)g];
-                const float4 f2 = feat[3 * (size_t)g + 2];
-                const Rect q = tile_rect(f0.x, f0.y, radius[g], B, tg.TX[v], tg.TY[v]);
-                if (w == 0) s_first = (int)(st[k] - base);
-                else w_start[w] = (uint16_t)(st[k] - base);
-                w_xy[w] = (uint32_t)q.x0 | ((uint32_t)q.y0 << 16);
-                w_wv[w] = (uint32_t)(q.x1 - q.x0) | ((uint32_t)v << 16);
-                w_g[w] = g;
-                w_m[w] = (unsigned long long)__float_as_uint(f2.y) |
-                         ((unsigned long long)__float_as_uint(f2.z) << 32);
-                top = w + 1;
-            }
-        }
-        if (top > 0) atomicMax(&s_nw, top);
-        __syncthreads();
-        const int nw = s_nw;
-        // each thread emits RS_IPT consecutive pairs: one search, then an incremental tile walk
-        static_assert(RS_IPT == 8, "the vector stores below write 8 pairs per thread");
-        const int rel0 = (int)threadIdx.x * RS_IPT;
-        const int nblock = (int)(end - base);
-        if (rel0 < nblock) {
-            int lo = 0, hi = nw - 1;  // the first staged Gaussian starts at or before 0 <= rel0
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;  // >= 1
-                if ((int)w_start[mid] <= rel0) lo = mid; else hi = mid - 1;
-            }
-            const int j = rel0 - (lo > 0 ? (int)w_start[lo] : s_first);
-            uint32_t wv = w_wv[lo];
-            int wx = (int)(wv & 0xffffu);
-            uint32_t xy = w_xy[lo];
-            uint32_t g = w_g[lo];
-            // with a tile mask, pair j is the j-th set bit (row-major, 8 bits per row)
-            unsigned long long mk = w_m[lo];
-            int tb = s_off[wv >> 16], TXv = s_tx[wv >> 16];
-            int next = lo + 1 < nw ? (int)w_start[lo + 1] : nblock;
-            int rx, ry;
-            if (mk) {
-                for (int c = 0; c < j; ++c) mk &= mk - 1;
-                const int b = __ffsll((long long)mk) - 1;
-                rx = b & 7; ry = b >> 3;
-            } else {
-                ry = j / wx; rx = j - ry * wx;
-            }
-            uint32_t kk[RS_IPT], vv[RS_IPT];
-            const int cnt = nblock - rel0 < RS_IPT ? nblock - rel0 : RS_IPT;
-#pragma unroll
-            for (int e = 0; e < RS_IPT; ++e) {
-                if (e < cnt) {
-                    if (rel0 + e >= next) {  // next Gaussian of the window
-                        ++lo;
-                        wv = w_wv[lo];
-                        wx = (int)(wv & 0xffffu); xy = w_xy[lo]; g = w_g[lo];
-                        mk = w_m[lo];
-                        tb = s_off[wv >> 16]; TXv = s_tx[wv >> 16];
-                        next = lo + 1 < nw ? (int)w_start[lo + 1] : nblock;
-                        if (mk) {
-                            const int b = __ffsll((long long)mk) - 1;
-                            rx = b & 7; ry = b >> 3;
-                        } else {
-                            rx = 0; ry = 0;
-                        }
-                    }
-                    uint32_t key = (uint32_t)(tb + ((int)(xy >> 16) + ry) * TXv + (int)(xy & 0xffffu) + rx);
-                    if (key >= n_tiles) {  // cannot happen for consistent inputs; never index past the grid
-                        *status = DG_ERR_CUDA;
-                        key = 0;
-                    }
-                    kk[e] = key;
-                    vv[e] = g;
-                    atomicAdd(&h[key & mask0], 1u);
-                    if (mk) {
-                        mk &= mk - 1;  // the next kept tile (none left when the Gaussian's pairs end)
-                        const int b = __ffsll((long long)mk) - 1;
-                        rx = b & 7; ry = b >> 3;
-                    } else if (++rx == wx) {
-                        rx = 0; ++ry;
-                    }
-                }
-            }
-            const long long i0 = base + rel0;
-            if (cnt == RS_IPT) {
-                uint4* kp = (uint4*)(pkey + i0);
-                uint4* vp = (uint4*)(pval + i0);
-                kp[0] = make_uint4(kk[0], kk[1], kk[2], kk[3]);
-                kp[1] = make_uint4(kk[4], kk[5], kk[6], kk[7]);
-                vp[0] = make_uint4(vv[0], vv[1], vv[2], vv[3]);
-                vp[1] = make_uint4(vv[4], vv[5], vv[6], vv[7]);
-            } else {
-                for (int e = 0; e < cnt; ++e) {
-                    pkey[i0 + e] = kk[e];
-                    pval[i0 + e] = vv[e];
-                }
-            }
+    // the column's digits, then the row's (a grid of one row or column has none there)
+    for (int part = 0; part < 2; ++part) {
+        const int b = part ? yb : k.xbits, n = (b + 7) / 8, from = part ? k.xbits : 0;
+        for (int i = 0, at = 0; i < n; ++i) {
+            const int w = (b - at + (n - i) - 1) / (n - i);
+            k.shift[k.npass] = from + at;
+            k.width[k.npass++] = w;
+            at += w;
         }
     }
-    __syncthreads();
-    for (int d = threadIdx.x; d <= (int)mask0; d += RS_THREADS) hist0[(long long)d * nblk + blockIdx.x] = h[d];
+    return k;
 }
 
-__global__ void k_ranges(const uint32_t* __restrict__ keys, const long long* M_dev, long long M_cap,
-                         uint2* __restrict__ ranges)
+// A record in depth order: rect corner x0 | y0 << 16, tile mask (or, with the
+// top bit of .w set, the rect's width and height), and its index in the view.
+constexpr uint32_t kRectFlag = 0x80000000u;
+
+// One tile of REC_TILE records of a view in depth order: gathers each one's
+// rect or tile mask, writes it and its first pair (relative to the view's
+// pairs), the record holding each pair tile's first pair, and the counts of the
+// lowest tile digit.  Also clears the range table.  Positions fit 32 bits: with
+// more pairs than M_cap (< 2^32) nothing is written.  The prefix comes first and
+// the digits are counted while the first warp looks back.
+__global__ void __launch_bounds__(OS_THREADS)
+k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const uint32_t* __restrict__ order,
+          long long P, int B, TileGrid tg, TileKey tk, Segs sg, const unsigned long long* __restrict__ npair,
+          long long M_cap, int pair_tile, const int* __restrict__ err1, BinCtl2* ctl, uint64_t* __restrict__ look,
+          uint4* __restrict__ rec, uint32_t* __restrict__ poff, uint32_t* __restrict__ bstart,
+          uint2* __restrict__ ranges)
 {
-    const long long M = eff_count(M_dev, M_cap);
-    const long long nq = (M + 3) / 4;
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < nq;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long i0 = 4 * q;
-        uint32_t k[4];
-        if (i0 + 3 < M) {
-            const uint4 v = *(const uint4*)(keys + i0);
-            k[0] = v.x; k[1] = v.y; k[2] = v.z; k[3] = v.w;
+    __shared__ int diff[OS_BINS];
+    __shared__ uint32_t direct[OS_BINS];
+    __shared__ uint32_t s_cycles;
+    __shared__ uint32_t ssum[OS_WARPS];
+    __shared__ uint32_t s_ex;
+    __shared__ long long s_tb;     // first pair tile of the view
+    __shared__ SegTile s_st;
+    __shared__ int s_dsum[OS_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_tiles = tg.off[tg.n];
+    for (long long i = (long long)blockIdx.x * OS_THREADS + threadIdx.x; i < n_tiles;
+         i += (long long)gridDim.x * OS_THREADS)
+        ranges[i] = make_uint2(0u, 0u);
+    if (warp == 0) {
+        uint32_t b = 0;
+        if (lane == 0) b = atomicAdd(&ctl->ctr[0], 1u);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        seg_tile(sg, b, REC_TILE, &s_st, lane);
+        __syncwarp();
+        const long long m = lane < sg.V ? (long long)npair[lane] : 0;
+        const long long mt = warp_incl_scan<long long>((m + pair_tile - 1) / pair_tile, lane) -
+                             (m + pair_tile - 1) / pair_tile;
+        if (lane == s_st.v) s_tb = mt;
+        const long long msum = __shfl_sync(0xffffffffu, warp_incl_scan<long long>(m, lane), 31);
+        __syncwarp();
+        if (lane == 0 && msum > M_cap) s_st.v = -1;  // too many pairs: nothing is emitted
+        if (lane == 0 && *err1 != 0) {               // the order is not complete: nothing is read by it
+            s_st.v = -1;
+            ctl->bad = 1;
+        }
+    }
+    diff[threadIdx.x] = 0;
+    direct[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_cycles = 0;
+    __syncthreads();
+    const SegTile st = s_st;
+    if (st.v < 0) return;
+    const int TX = tg.TX[st.v], TY = tg.TY[st.v];
+    const long long m_view = (long long)npair[st.v];
+    const long long first = (long long)st.t * REC_TILE + warp * (32 * REC_IPT) + lane;  // position in the view
+    const uint32_t* ord = order + st.off;
+    uint32_t r[REC_IPT];
+#pragma unroll
+    for (int k = 0; k < REC_IPT; ++k) r[k] = first + 32 * k < st.n ? ord[first + 32 * k] : 0u;
+    float2 uv[REC_IPT];
+    float4 f2[REC_IPT];
+    int rad[REC_IPT];
+#pragma unroll
+    for (int k = 0; k < REC_IPT; ++k) {
+        const float4* f = feat + 3 * (size_t)r[k];
+        uv[k] = *(const float2*)f;
+        f2[k] = f[2];
+        rad[k] = radius[r[k]];
+    }
+    uint32_t cnt[REC_IPT], ex[REC_IPT];
+    uint4 out[REC_IPT];
+    uint32_t run = 0;
+#pragma unroll
+    for (int k = 0; k < REC_IPT; ++k) {
+        const Rect q = tile_rect(uv[k].x, uv[k].y, rad[k], B, TX, TY);
+        const uint32_t mlo = __float_as_uint(f2[k].y), mhi = __float_as_uint(f2[k].z);
+        const uint32_t w = (uint32_t)(q.x1 - q.x0), h = (uint32_t)(q.y1 - q.y0);
+        const bool masked = (mlo | mhi) != 0;
+        out[k] = make_uint4((uint32_t)q.x0 | ((uint32_t)q.y0 << 16), masked ? mlo : w, masked ? mhi : h,
+                            (uint32_t)(r[k] - (uint32_t)(st.v * P)) | (masked ? 0u : kRectFlag));
+        cnt[k] = first + 32 * k < st.n ? (masked ? (uint32_t)(__popc(mlo) + __popc(mhi)) : w * h) : 0u;
+        const uint32_t inc = warp_incl_scan<uint32_t>(cnt[k], lane);
+        ex[k] = run + inc - cnt[k];
+        run += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    if (lane == 0) ssum[warp] = run;
+    __syncthreads();
+    uint32_t pre = 0, tot = 0;
+#pragma unroll
+    for (int w = 0; w < OS_WARPS; ++w) {
+        pre += w < warp ? ssum[w] : 0u;
+        tot += ssum[w];
+    }
+    if (warp == 0) {
+        uint64_t* lk = look + st.tbase + st.t;
+        if (lane == 0) st_relaxed(lk, (st.t == 0 ? kLbInc : kLbAgg) | tot);
+        uint64_t e = 0;
+        if (st.t > 0) {
+            if (!os_lookback_warp(lk - st.t, st.t, &e, lane)) {
+                if (lane == 0) atomicExch(&ctl->err, DG_ERR_TIMEOUT);
+                ctl->bad = 1;
+            }
+            if (lane == 0) st_relaxed(lk, kLbInc | ((e + tot) & kLbCount));
+        }
+        if (lane == 0) {
+            s_ex = (uint32_t)e;
+            // (cannot differ for the depths, tiles, records and radii of one projection)
+            if ((long long)(st.t + 1) * REC_TILE >= st.n && (long long)(e + tot) != m_view) {
+                atomicCAS(&ctl->err, 0, DG_ERR_CUDA);
+                ctl->bad = 1;
+            }
+        }
+    }
+    // counts of the lowest digit (or of the whole key, when it is one digit)
+    const uint32_t dm = (1u << tk.width[0]) - 1u;
+#pragma unroll
+    for (int k = 0; k < REC_IPT; ++k) {
+        if (cnt[k] == 0) continue;
+        const uint32_t x0 = out[k].x & 0xffffu, y0 = out[k].x >> 16;
+        const bool masked = !(out[k].w & kRectFlag);
+        if (tk.npass == 1) {
+            const uint32_t k0 = (y0 << tk.xbits) + x0;
+            if (masked) {
+                unsigned long long mk = (unsigned long long)out[k].y | ((unsigned long long)out[k].z << 32);
+#pragma unroll 1
+                for (; mk; mk &= mk - 1) {
+                    const uint32_t b = (uint32_t)__ffsll((long long)mk) - 1u;
+                    atomicAdd(&direct[(k0 + ((b >> 3) << tk.xbits) + (b & 7u)) & dm], 1u);
+                }
+            } else {
+#pragma unroll 1
+                for (uint32_t y = 0; y < out[k].z; ++y) {
+                    const uint32_t a = k0 + (y << tk.xbits), e = a + out[k].y;
+                    atomicAdd(&diff[a & dm], 1);
+                    if (e <= dm) atomicAdd(&diff[e], -1);
+                }
+            }
+        } else if (masked) {
+            // pairs of each of the mask's eight columns
+            uint32_t any = out[k].y | out[k].z;
+            any |= any >> 16;
+            any = (any | (any >> 8)) & 255u;
+#pragma unroll 1
+            for (; any; any &= any - 1) {
+                const int c = __ffs((int)any) - 1;
+                const uint32_t col = 0x01010101u << c;
+                atomicAdd(&direct[(x0 + c) & dm], (uint32_t)(__popc(out[k].y & col) + __popc(out[k].z & col)));
+            }
         } else {
-            for (int c = 0; c < 4; ++c) k[c] = i0 + c < M ? keys[i0 + c] : 0xffffffffu;
-        }
-        uint32_t prev = i0 > 0 ? keys[i0 - 1] : 0xffffffffu;
-        const uint32_t next = i0 + 4 < M ? keys[i0 + 4] : 0xffffffffu;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const long long i = i0 + c;
-            if (i >= M) break;
-            const uint32_t nx = c < 3 ? k[c + 1] : next;
-            if (i == 0 || prev != k[c]) ranges[k[c]].x = (uint32_t)i;
-            if (i == M - 1 || nx != k[c]) ranges[k[c]].y = (uint32_t)(i + 1);
-            prev = k[c];
+            // columns x0 .. x0 + w - 1, each h times: cyclic through the digit's values
+            const uint32_t w = out[k].y, h = out[k].z, rem = w & dm, lo = x0 & dm, hi = lo + rem;
+            if (w > dm) atomicAdd(&s_cycles, (w >> tk.width[0]) * h);
+            if (rem) {
+                atomicAdd(&diff[lo], (int)h);
+                if (hi != dm + 1u) atomicAdd(&diff[hi & dm], -(int)h);
+                if (hi > dm + 1u) atomicAdd(&diff[0], (int)h);
+            }
         }
     }
+    __syncthreads();
+    const int mine = diff[threadIdx.x];
+    const int dinc = warp_incl_scan<int>(mine, lane);
+    if (lane == 31) s_dsum[warp] = dinc;
+    __syncthreads();
+    uint32_t c0 = (uint32_t)dinc + s_cycles + direct[threadIdx.x];
+#pragma unroll
+    for (int w = 0; w < OS_WARPS; ++w) c0 += w < warp ? (uint32_t)s_dsum[w] : 0u;
+    if (threadIdx.x <= dm && c0) atomicAdd(&ctl->hist[st.v][0][threadIdx.x], c0);
+    pre += s_ex;
+#pragma unroll
+    for (int k = 0; k < REC_IPT; ++k) {
+        const long long s = first + 32 * k;
+        if (s >= st.n) continue;
+        const uint32_t a = pre + ex[k];
+        rec[st.off + s] = out[k];
+        poff[st.off + s] = a;
+        const long long e = (long long)a + cnt[k];
+        for (long long b = ((long long)a + pair_tile - 1) / pair_tile; b * pair_tile < e && b * pair_tile < m_view; ++b)
+            bstart[s_tb + b] = (uint32_t)s;
+    }
+}
+
+// First tile pass: the pairs of its tile, formed from the records in depth
+// order.  A thread takes a record and writes its pairs to their places in
+// shared memory (tile mask: a walk over the set bits, at most 64); the rects
+// without a mask, of any size, are written by the whole warp, 32 pairs at a
+// time.  (One thread per 16 consecutive pairs, walking along the records, left
+// 16-way bank conflicts and a chain of dependent record loads.  A warp-round
+// of 32 records takes about 240 instructions; issue and the pass behind it bound
+// the kernel: 96 us on 5.9M pairs.)
+struct SrcEmit {
+    const uint4* rec;
+    const uint32_t* poff;
+    const uint32_t* bstart;
+    const unsigned long long* nvis;
+    long long P;
+    TileGrid tg;
+    int xbits;
+    BinCtl2* ctl;
+    template <int IPT>
+    __device__ __forceinline__ uint32_t load(const SegTile& st, int nv, uint32_t* sk, uint32_t* sv,
+                                             uint32_t (&key)[IPT], int warp, int lane) const
+    {
+        constexpr int TILE = OS_THREADS * IPT;
+        const uint32_t base = st.t * (uint32_t)TILE;  // first pair (relative to the view's)
+        const uint4* rv = rec + st.v * P;
+        const uint32_t* pv = poff + st.v * P;
+        const uint32_t s_lo = bstart[st.tbase + st.t];
+        const uint32_t s_hi = (long long)base + TILE < st.n ? bstart[st.tbase + st.t + 1] : (uint32_t)nvis[st.v] - 1u;
+        const int nr = (int)(s_hi - s_lo) + 1;
+        const uint32_t row = 1u << xbits;
+        const uint32_t n_keys = (uint32_t)tg.TY[st.v] << xbits;
+        const uint32_t rbase = (uint32_t)(st.v * P);
+        bool bad = false;
+        // (whole warps step together: the last round's idle lanes hold an empty mask)
+        for (int i0 = warp * 32; i0 < nr; i0 += OS_THREADS) {
+            const bool on = i0 + lane < nr;
+            const uint32_t s = s_lo + (uint32_t)(on ? i0 + lane : 0);
+            const uint4 c = rv[s];
+            const int p0 = (int)(pv[s] - base);  // of the record's first pair in this tile's array (may be negative)
+            const bool whole = on && (c.w & kRectFlag) != 0;
+            const uint32_t g = rbase + (c.w & ~kRectFlag);
+            const uint32_t k0 = (c.x >> 16) * row + (c.x & 0xffffu);
+            // the mask's two words in turn (most masks have no bit above the fourth tile row)
+            int p = p0;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t mk = on && !whole ? (half ? c.z : c.y) : 0u;
+                const uint32_t kh = k0 + 4u * half * row;
+#pragma unroll 1
+                for (; mk; ++p, mk &= mk - 1) {
+                    const uint32_t b = (uint32_t)__ffs((int)mk) - 1u;
+                    const uint32_t kk = kh + (b >> 3) * row + (b & 7u);
+                    if ((uint32_t)p < (uint32_t)nv) {
+                        bad = bad || kk >= n_keys;
+                        sk[p] = kk < n_keys ? kk : 0u;
+                        sv[p] = g;
+                    }
+                }
+            }
+            uint32_t todo = __ballot_sync(0xffffffffu, whole);
+            while (todo) {
+                const int l = __ffs((int)todo) - 1;
+                todo &= todo - 1;
+                const int q0 = __shfl_sync(0xffffffffu, p0, l);
+                const uint32_t w = __shfl_sync(0xffffffffu, c.y, l), h = __shfl_sync(0xffffffffu, c.z, l);
+                const uint32_t kb = __shfl_sync(0xffffffffu, k0, l), gg = __shfl_sync(0xffffffffu, g, l);
+                const int a = q0 < 0 ? 0 : q0;
+                const long long end = (long long)q0 + (long long)w * h;
+                const int e = end < nv ? (int)end : nv;
+                for (int i = a + lane; i < e; i += 32) {
+                    const uint32_t j = (uint32_t)(i - q0), y = j / w;
+                    const uint32_t kk = kb + y * row + (j - y * w);
+                    bad = bad || kk >= n_keys;
+                    sk[i] = kk < n_keys ? kk : 0u;
+                    sv[i] = gg;
+                }
+            }
+        }
+        // (cannot happen for consistent inputs; no key leaves the grid)
+        if (bad) atomicCAS(&ctl->err, 0, DG_ERR_CUDA);
+        __syncthreads();
+        const int seg = warp * 32 * IPT + lane;
+        uint32_t ok = 0;
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) {
+            const bool in = seg + 32 * i < nv;
+            key[i] = in ? sk[seg + 32 * i] : 0u;
+            ok |= (in ? 1u : 0u) << i;
+        }
+        return ok;
+    }
+    template <int IPT>
+    __device__ __forceinline__ void values(const SegTile&, int nv, const uint32_t* sv, uint32_t (&val)[IPT], int warp,
+                                           int lane) const
+    {
+        const int seg = warp * 32 * IPT + lane;
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) val[i] = seg + 32 * i < nv ? sv[seg + 32 * i] : 0u;
+    }
+};
+
+// Ranges from their (complement of the start, end) form, and the call's status.
+__global__ void k_ranges_final(uint2* __restrict__ ranges, int n_tiles, const long long* M, long long M_cap,
+                               const int* err1, const BinCtl2* ctl, int* status)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n_tiles) {
+        const uint2 r = ranges[i];
+        if (r.y != 0u) ranges[i].x = ~r.x;
+    }
+    if (i == 0) *status = *M > M_cap ? DG_ERR_CAPACITY : (*err1 != 0 ? *err1 : ctl->err);
 }
 
 // Workspace layout (offsets 256-byte aligned).  The pair count and the
-// P-sized buffers come first so that their offsets do not depend on M_cap:
-// phase 1 and phase 2 may be called with workspaces laid out for different
-// capacities as long as the P part was carried over.
+// record-sized buffers come first so that their offsets do not depend on
+// M_cap: phase 1 and phase 2 may be called with workspaces laid out for
+// different capacities as long as the record part was carried over.
 struct BinWs {
     long long* M;                       // total pair count
-    uint32_t *dk0, *dv0, *dk1, *dv1;   // depth sort, P each
-    uint64_t* poff;                     // P pair offsets
-    OsCtl* ctl1;                        // phase 1 control block, then the scan's look-back words
-    uint64_t* slook;
-    size_t ctl1_bytes;                  // bytes phase 1 clears from ctl1 on
-    uint64_t* look[2];                  // phase 1 radix look-back words, alternating between passes
+    BinCtl1* ctl1;                      // phase 1 control block, then its look-back words
+    void* look1;                        // [4][tiles][256]
+    size_t look1_pass;                  // bytes of one pass
+    size_t zero1;                       // bytes phase 1 clears from ctl1 on
+    uint32_t *dk0, *dv0, *dk1, *dv1;   // depth sort, N each
+    uint4* rec;                         // records in depth order, N (over dk0, dk1 and two more words per record)
+    uint32_t* poff;                     // N first pairs
+    BinCtl2* ctl2;                      // phase 2 control block, then its look-back words
+    uint64_t* rlook;                    // records scan
+    void* look2;                        // [BIN_MAXPASS][pair tiles][256], 2^width words of a tile used
+    size_t zero2_fixed;                 // bytes phase 2 clears from ctl2 up to look2
     uint32_t *pk0, *pv0, *pk1, *pv1;   // pair sort, M_cap each
-    uint32_t* pkfin;                    // sorted pair keys, M_cap
-    int* bstart;                        // first sorted position of each pair block
-    uint32_t* hist;                     // phase 2 per-block digit counts
-    uint64_t* bsum;                     // phase 2 scan block sums
+    uint32_t* bstart;                   // record holding each pair tile's first pair
     size_t bytes;
 };
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-static BinWs bin_layout(char* base, long long P, long long M_cap)
+// Items per thread of a pass over at most n items, and the look-back word size.
+static int os_ipt(long long n) { return n <= OS_SMALL_MAX ? OS_IPT_SMALL : OS_IPT_BIG; }
+static size_t os_word(long long n) { return n < (1ll << 30) ? 4 : 8; }
+// Tiles of `views` segments holding n items together (each ends in a partial tile).
+static long long os_tiles(long long n, int views, int tile) { return n / tile + views; }
+
+static BinWs bin_layout(char* base, long long P, int n_views, long long M_cap)
 {
+    const long long N = P * n_views;
     BinWs w;
     size_t o = 0;
     auto take = [&](size_t bytes) { char* p = base + o; o += align256(bytes); return p; };
     w.M = (long long*)take(8);
-    w.dk0 = (uint32_t*)take(4 * P); w.dv0 = (uint32_t*)take(4 * P);
-    w.dk1 = (uint32_t*)take(4 * P); w.dv1 = (uint32_t*)take(4 * P);
-    w.poff = (uint64_t*)take(8 * P);
-    const size_t c0 = o;
-    w.ctl1 = (OsCtl*)take(sizeof(OsCtl));
-    w.slook = (uint64_t*)take(8 * ((P + SCAN_TILE - 1) / SCAN_TILE + 1));
-    w.ctl1_bytes = o - c0;
-    const long long nlook = (P + RS_TILE - 1) / RS_TILE * (1 << RS_MAXBITS);
-    w.look[0] = (uint64_t*)take(8 * nlook);
-    w.look[1] = (uint64_t*)take(8 * nlook);
+    const size_t c1 = o;
+    w.ctl1 = (BinCtl1*)take(sizeof(BinCtl1));
+    w.look1_pass = align256(os_word(N) * OS_BINS * (size_t)os_tiles(N, n_views, OS_THREADS * os_ipt(N)));
+    w.look1 = take(4 * w.look1_pass);
+    w.zero1 = o - c1;
+    w.dk0 = (uint32_t*)take(4 * N); w.dv0 = (uint32_t*)take(4 * N);
+    w.dk1 = (uint32_t*)take(4 * N); w.dv1 = (uint32_t*)take(4 * N);
+    w.rec = (uint4*)take(16 * N);
+    w.poff = (uint32_t*)take(4 * N);
+    const size_t c2 = o;
+    w.ctl2 = (BinCtl2*)take(sizeof(BinCtl2));
+    w.rlook = (uint64_t*)take(8 * os_tiles(N, n_views, REC_TILE));
+    w.zero2_fixed = o - c2;
+    // (from here on the offsets depend on M_cap)
+    const long long pt = os_tiles(M_cap, n_views, OS_THREADS * os_ipt(M_cap));
+    w.look2 = take(BIN_MAXPASS * align256(os_word(M_cap) * OS_BINS * pt));
     w.pk0 = (uint32_t*)take(4 * M_cap); w.pv0 = (uint32_t*)take(4 * M_cap);
     w.pk1 = (uint32_t*)take(4 * M_cap); w.pv1 = (uint32_t*)take(4 * M_cap);
-    w.pkfin = (uint32_t*)take(4 * M_cap);
-    w.bstart = (int*)take(4 * ((M_cap + RS_TILE - 1) / RS_TILE + 1));
-    const long long nblk = (M_cap + RS_TILE - 1) / RS_TILE;
-    const long long nh = (long long)(1 << RS_MAXBITS) * nblk;
-    w.hist = (uint32_t*)take(4 * nh);
-    const long long nscan = (nh > M_cap ? nh : M_cap);
-    w.bsum = (uint64_t*)take(8 * ((nscan + SCAN_TILE - 1) / SCAN_TILE + 1));
+    w.bstart = (uint32_t*)take(4 * (pt + 1));
     w.bytes = o;
     return w;
 }
 
-// Where phase 1 leaves the (view, depth, index) order of the records.
-static uint32_t* order_buffer(const BinWs& w, int n_views) { return n_views > 1 ? w.dv1 : w.dv0; }
-
-static int view_bits(int n_views)
+// One pass over at most n_max items; the kernel's form by the item count.
+template <int NB, class Src>
+static void os_pass(const Src& src, const Segs& sg, const OsPass& ps, long long n_max, cudaStream_t s)
 {
-    int b = 0;
-    while ((1 << b) < n_views) ++b;
-    return b;
+    const int ipt = os_ipt(n_max);
+    const int grid = (int)os_tiles(n_max, sg.V, OS_THREADS * ipt);
+    if (ipt == OS_IPT_SMALL) k_os_pass<OS_IPT_SMALL, uint32_t, NB><<<grid, OS_THREADS, 0, s>>>(src, sg, ps);
+    else if (os_word(n_max) == 4) k_os_pass<OS_IPT_BIG, uint32_t, NB><<<grid, OS_THREADS, 0, s>>>(src, sg, ps);
+    else k_os_pass<OS_IPT_BIG, uint64_t, NB><<<grid, OS_THREADS, 0, s>>>(src, sg, ps);
+    dg_note_launch();
 }
 
 }  // namespace dg
@@ -381,7 +556,7 @@ static int view_bits(int n_views)
 extern "C" size_t dg_bin_workspace_size(int64_t P, int32_t n_views, int64_t M_cap)
 {
     if (P < 0 || M_cap < 0 || n_views < 1 || n_views > DG_MAX_VIEWS) return 0;
-    return dg::bin_layout(nullptr, P * n_views, M_cap).bytes;
+    return dg::bin_layout(nullptr, P, n_views, M_cap).bytes;
 }
 
 extern "C" dg_status dg_bin_count(const float* depth, const int32_t* tiles, int64_t P, int32_t n_views, void* ws,
@@ -394,54 +569,48 @@ extern "C" dg_status dg_bin_count(const float* depth, const int32_t* tiles, int6
     }
     if (!ws || !M_out || (P > 0 && (!depth || !tiles))) { dg_set_error("null buffer"); return DG_ERR_ARG; }
     const long long N = P * n_views;
-    const dg::BinWs w = dg::bin_layout((char*)ws, N, M_cap);
+    const dg::BinWs w = dg::bin_layout((char*)ws, P, n_views, M_cap);
     if (ws_bytes < w.bytes) { dg_set_error("workspace %zu < %zu bytes", ws_bytes, w.bytes); return DG_ERR_CAPACITY; }
     cudaStream_t s = (cudaStream_t)stream;
-    cudaMemsetAsync(w.ctl1, 0, w.ctl1_bytes, s);  // counters, error word, scan look-back
+    cudaMemsetAsync(w.ctl1, 0, w.zero1, s);  // counters, error word, look-back words
     if (N == 0) {
         cudaMemsetAsync(w.M, 0, sizeof(long long), s);
         cudaMemsetAsync(M_out, 0, sizeof(long long), s);
         return dg_check_launch("bin_count");
     }
     using namespace dg;
-    const int vb = n_views > 1 ? view_bits(n_views + 1) : 0;
-    const int npass = vb > 0 ? 5 : 4;
-    const long long ntile = (N + RS_TILE - 1) / RS_TILE;
-    const int hb = (int)(ntile < 152 * 4 ? ntile : 152 * 4);
-    k_os_hist_depth<<<hb, RS_THREADS, 0, s>>>(depth, tiles, N, (uint32_t)P, (uint32_t)n_views, vb, w.ctl1,
-                                              w.look[0]);
-    k_os_base<<<1, 256, 0, s>>>(w.ctl1, npass);
-    dg_note_launch(2);
-    // 4 depth passes: (depth, index) -> 1 -> 0 -> 1 -> values only in dv0;
-    // then the view pass dv0 -> dv1 (order_buffer tells which holds the result)
-    auto pass = [&](int p, int bits) {
-        OsPass ps;
-        ps.look = w.look[p & 1];
-        ps.look_next = p + 1 < npass ? w.look[(p + 1) & 1] : nullptr;
-        ps.next_nbins = p + 1 < npass ? (p + 1 < 4 ? 256 : 1 << vb) : 0;
+    const long long per_block = DH_THREADS * DH_IPT;
+    long long hb = (P + per_block - 1) / per_block;
+    const long long hmax = (152 * 4 + n_views - 1) / n_views;
+    if (hb > hmax) hb = hmax;
+    k_depth_hist<<<dim3((unsigned)hb, (unsigned)n_views), DH_THREADS, 0, s>>>(depth, tiles, P, w.ctl1);
+    dg_note_launch();
+    // depth passes: (depth, record) -> 1 -> 0 -> 1 -> records only in dv0
+    auto pass = [&](int p, uint32_t* ko, uint32_t* vo) {
+        OsPass ps{};
+        ps.look = (char*)w.look1 + p * w.look1_pass;
         ps.ctr = &w.ctl1->ctr[p];
-        ps.base = w.ctl1->base[p];
+        ps.hist = &w.ctl1->hist[0][p][0];
+        ps.hist_stride = 4 * OS_BINS;
         ps.err = &w.ctl1->err;
-        ps.shift = p < 4 ? 8 * p : 0;
-        ps.mask = (1u << bits) - 1u;
+        ps.shift = 8 * p;
+        ps.mask = OS_BINS - 1;
+        ps.kout = ko;
+        ps.vout = vo;
+        if (p == 0) {
+            ps.m_views = w.ctl1->npair;
+            ps.m_ws = w.M;
+            ps.m_out = (long long*)M_out;
+        }
         return ps;
     };
-    const int nblk = (int)ntile;
-    k_os_pass<<<nblk, RS_THREADS, 0, s>>>(SrcDepth{depth, tiles}, w.dk1, w.dv1, nullptr, N, pass(0, 8));
-    k_os_pass<<<nblk, RS_THREADS, 0, s>>>(SrcKV{w.dk1, w.dv1}, w.dk0, w.dv0, nullptr, N, pass(1, 8));
-    k_os_pass<<<nblk, RS_THREADS, 0, s>>>(SrcKV{w.dk0, w.dv0}, w.dk1, w.dv1, nullptr, N, pass(2, 8));
-    k_os_pass<<<nblk, RS_THREADS, 0, s>>>(SrcKV{w.dk1, w.dv1}, nullptr, w.dv0, nullptr, N, pass(3, 8));
-    dg_note_launch(4);
-    if (vb > 0) {
-        k_os_pass<<<nblk, RS_THREADS, 0, s>>>(SrcView{w.dv0, tiles, (uint32_t)P, (uint32_t)n_views}, nullptr,
-                                              w.dv1, nullptr, N, pass(4, vb));
-        dg_note_launch();
-    }
-    const int sb = (int)((N + SCAN_TILE - 1) / SCAN_TILE);
-    k_os_scan<<<sb, SCAN_THREADS, 0, s>>>(LoadTilesInOrder{tiles, order_buffer(w, n_views)}, N, w.poff, w.slook,
-                                          &w.ctl1->ctr[OS_MAXPASS - 1], w.M, &w.ctl1->err);
-    dg_note_launch();
-    cudaMemcpyAsync(M_out, w.M, sizeof(long long), cudaMemcpyDeviceToDevice, s);
+    const Segs all{n_views, nullptr, P, P, LLONG_MAX, nullptr};
+    const Segs vis{n_views, w.ctl1->nvis, 0, P, LLONG_MAX, nullptr};
+    os_pass<8>(SrcDepth{depth, tiles}, all, pass(0, w.dk1, w.dv1), N, s);
+    os_pass<8>(SrcKV{w.dk1, w.dv1}, vis, pass(1, w.dk0, w.dv0), N, s);
+    os_pass<8>(SrcKV{w.dk0, w.dv0}, vis, pass(2, w.dk1, w.dv1), N, s);
+    // (the highest digit, sign and upper exponent bits, has few distinct values)
+    os_pass<0>(SrcKV{w.dk1, w.dv1}, vis, pass(3, nullptr, w.dv0), N, s);
     return dg_check_launch("bin_count");
 }
 
@@ -461,48 +630,72 @@ extern "C" dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64
         dg_set_error("null buffer");
         return DG_ERR_ARG;
     }
+    using namespace dg;
     const long long N = P * n_views;
-    const dg::BinWs w = dg::bin_layout((char*)ws, N, M_cap);
+    const BinWs w = bin_layout((char*)ws, P, n_views, M_cap);
     if (ws_bytes < w.bytes) { dg_set_error("workspace %zu < %zu bytes", ws_bytes, w.bytes); return DG_ERR_CAPACITY; }
-    dg::TileGrid tg;
+    TileGrid tg;
     tg.n = n_views;
-    long long n_tiles = 0;
+    long long n_tiles = 0, most = 1;
     for (int v = 0; v < n_views; ++v) {
         tg.TX[v] = (cams[v].width + tile - 1) / tile;
         tg.TY[v] = (cams[v].height + tile - 1) / tile;
         tg.off[v] = (int)n_tiles;
-        n_tiles += (long long)tg.TX[v] * tg.TY[v];
+        const long long nt = (long long)tg.TX[v] * tg.TY[v];
+        n_tiles += nt;
+        if (nt > most) most = nt;
     }
     tg.off[n_views] = (int)n_tiles;
     if (n_tiles > (1ll << 30)) { dg_set_error("too many tiles"); return DG_ERR_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
-    cudaMemsetAsync(ranges, 0, sizeof(uint32_t) * 2 * n_tiles, s);
-    cudaMemsetAsync(status, 0, sizeof(int32_t), s);
-    int bits = 0;
-    while ((1ll << bits) < n_tiles) ++bits;
-    const int b0 = dg::first_pass_bits(bits);
-    const uint32_t mask0 = b0 > 0 ? (1u << b0) - 1u : 0u;
-    const int nblk = (int)((M_cap + dg::RS_TILE - 1) / dg::RS_TILE);
-    const int pb = (int)((N + 255) / 256);
-    uint32_t* order = dg::order_buffer(w, n_views);
-    if (N > 0 && nblk > 0) {
-        dg::k_block_starts<<<pb, 256, 0, s>>>(w.poff, N, w.M, M_cap, w.bstart);
+    const TileKey tk = tile_key(tg);
+    const int ipt = os_ipt(M_cap);
+    const int pair_tile = OS_THREADS * ipt;
+    size_t look_at[BIN_MAXPASS + 1] = {0};
+    for (int p = 0; p < tk.npass; ++p)
+        look_at[p + 1] = look_at[p] + align256((os_word(M_cap) << tk.width[p]) * (size_t)os_tiles(M_cap, n_views, pair_tile));
+    if (N > 0 && M_cap > 0) {
+        cudaMemsetAsync(w.ctl2, 0, w.zero2_fixed + look_at[tk.npass], s);
+        const Segs vis{n_views, w.ctl1->nvis, 0, P, LLONG_MAX, nullptr};
+        k_records<<<(int)os_tiles(N, n_views, REC_TILE), OS_THREADS, 0, s>>>(
+            (const float4*)feat, radius, w.dv0, P, tile, tg, tk, vis, w.ctl1->npair, M_cap, pair_tile,
+            &w.ctl1->err, w.ctl2, w.rlook, w.rec, w.poff, w.bstart, (uint2*)ranges);
         dg_note_launch();
+        const Segs pairs{n_views, w.ctl1->npair, 0, -1, M_cap, &w.ctl2->bad};
+        uint32_t *ki = nullptr, *vi = nullptr;
+        for (int p = 0; p < tk.npass; ++p) {
+            const bool last = p == tk.npass - 1;
+            uint32_t* ko = last ? nullptr : (p & 1) ? w.pk1 : w.pk0;
+            uint32_t* vo = last ? gid : (p & 1) ? w.pv1 : w.pv0;
+            OsPass ps{};
+            ps.look = (char*)w.look2 + look_at[p];
+            ps.ctr = &w.ctl2->ctr[1 + p];
+            ps.hist = &w.ctl2->hist[0][p][0];
+            ps.hist_stride = BIN_MAXPASS * OS_BINS;
+            ps.err = &w.ctl2->err;
+            ps.shift = tk.shift[p];
+            ps.mask = (1u << tk.width[p]) - 1u;
+            ps.kout = ko;
+            ps.vout = vo;
+            ps.hist_next = last ? nullptr : &w.ctl2->hist[0][p + 1][0];
+            ps.mask_next = last ? 0u : (1u << tk.width[p + 1]) - 1u;
+            if (last) {
+                ps.xbits = tk.xbits;
+                for (int v = 0; v < n_views; ++v) ps.TX[v] = tg.TX[v];
+                ps.ranges = (uint2*)ranges;
+                for (int v = 0; v <= n_views; ++v) ps.toff[v] = tg.off[v];
+            }
+            if (p == 0) os_pass<8>(SrcEmit{w.rec, w.poff, w.bstart, w.ctl1->nvis, P, tg, tk.xbits, w.ctl2}, pairs, ps, M_cap, s);
+            else os_pass<8>(SrcKV{ki, vi}, pairs, ps, M_cap, s);
+            ki = ko;
+            vi = vo;
+        }
+    } else {
+        cudaMemsetAsync(w.ctl2, 0, sizeof(BinCtl2), s);
+        cudaMemsetAsync(ranges, 0, sizeof(uint32_t) * 2 * n_tiles, s);
     }
-    // emit pairs in (view, depth) order (slots from phase 1) with pass-0 histogram, or flag overflow
-    dg::k_emit<<<nblk > 0 ? nblk : 1, dg::RS_THREADS, 0, s>>>((const float4*)feat, radius, order, w.poff, w.bstart,
-                                                            N, (uint32_t)(P > 0 ? P : 1), w.M, M_cap, tile, tg, mask0,
-                                                            w.pk0, w.pv0, w.hist, nblk > 0 ? nblk : 1, &w.ctl1->err,
-                                                            status);
-    dg_note_launch();
-    if (M_cap == 0) return dg_check_launch("bin_sort");
-    dg::SortBufs sb{w.hist, w.bsum};
-    dg::radix_sort(w.pk0, w.pv0, w.pk1, w.pv1, w.pkfin, gid, w.M, M_cap, bits, sb, s, /*hist0_ready=*/bits > 0,
-                   dg::kTileBallotPasses);
-    const long long nq = (M_cap + 3) / 4;
-    long long rb = (nq + 255) / 256;
-    if (rb > 152 * 32) rb = 152 * 32;
-    dg::k_ranges<<<(int)(rb > 0 ? rb : 1), 256, 0, s>>>(w.pkfin, w.M, M_cap, (uint2*)ranges);
+    k_ranges_final<<<(int)((n_tiles + 255) / 256), 256, 0, s>>>((uint2*)ranges, (int)n_tiles, w.M, M_cap,
+                                                              &w.ctl1->err, w.ctl2, status);
     dg_note_launch();
     return dg_check_launch("bin_sort");
 }
