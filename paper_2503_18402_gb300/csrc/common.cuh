@@ -147,6 +147,36 @@ __device__ inline bool tile_skip(const float4& a, const float4& b, float px0, fl
     return fmin > 2.f * __logf(255.f * o) + 0.02f;
 }
 
+// tile_skip for the 8x4 blocks of the warp-per-block render passes, with
+// log2(o) given and only the rectangle's edges that face the Gaussian's centre:
+// along a ray from the centre the form grows with the square of the distance,
+// so a point of a rectangle that does not hold the centre has a smaller value
+// in front of it, where its ray enters through such an edge.
+__device__ __forceinline__ bool block_skip(const float4& a, const float4& b, float log2o, float px0, float px1, float py0,
+                                           float py1)
+{
+    const float dxl = a.x - px1, dxh = a.x - px0, dyl = a.y - py1, dyh = a.y - py0;
+    const float A = a.z, B = a.w, C = b.x;
+    float best = 3.4e38f;
+    const bool outx = dxl > 0.f || dxh < 0.f, outy = dyl > 0.f || dyh < 0.f;
+    if (!outx && !outy) best = 0.f;
+    const float ex = dxl > 0.f ? dxl : dxh, ey = dyl > 0.f ? dyl : dyh;
+    // (the minimiser on an edge only has to be near: the form is flat there)
+    const float fy = fminf(fmaxf(__fdividef(-B * ex, C), dyl), dyh);
+    const float fx = fminf(fmaxf(__fdividef(-B * ey, A), dxl), dxh);
+    {
+        const float s = A * ex * ex, t = 2.f * B * ex * fy, u = C * fy * fy;
+        if (outx) best = (s + t + u) - 1e-5f * (s + fabsf(t) + u);
+    }
+    {
+        const float s = A * fx * fx, t = 2.f * B * fx * ey, u = C * ey * ey;
+        if (outy) best = fminf(best, (s + t + u) - 1e-5f * (s + fabsf(t) + u));
+    }
+    // alpha = o exp(-best/2) < 1/255  <=>  best > 2 ln(255 o); 0.02 absorbs the
+    // per-pixel rounding of the power and of exp
+    return !(b.y >= kAlphaMin) || best > fmaf(1.3862943611198906f, log2o, 11.082527f + 0.02f);
+}
+
 // Two float32 values in one 64-bit register for the packed float32 operations
 // of sm_100 and later (PTX .f32x2): one instruction does the operation on both
 // halves, each rounded exactly as the scalar operation (fma: one rounding), so
@@ -185,9 +215,6 @@ __device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b)
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-
-// The two floats at x (8-byte aligned) as one packed register.
-__device__ __forceinline__ f32x2 f2_ld(const float& x) { return *(const f32x2*)&x; }
 
 }  // namespace dg
 
