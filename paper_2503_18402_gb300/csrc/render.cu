@@ -860,8 +860,10 @@ k_render_bwd(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
     }  // work items
 }
 
-constexpr int kEpG = 16;
-constexpr int kEpPitch = 33;  // float2 per entry row of the (entry, pixel) matrix: 32 pixels + 1
+constexpr int kEpG = 16;                      // entries per group
+constexpr int kEpRing = 48;                   // staged entries: a group less one, and a batch of 32
+constexpr int kEpPitch = 33;                  // float4 per entry pair of the (pair, pixel) matrix: 32 pixels + 1
+constexpr int kPairW = 5;                     // float4 per staged entry pair
 
 // Next work item of this warp: item index w covers tile (or chunk) w / 2 and
 // the 8x4 pixel block w % 2 of it; *blk receives the block.  Warp-uniform.
@@ -889,34 +891,53 @@ __device__ inline Item next_item_warp(int* counter, int count, const int4* list,
     return it;
 }
 
+// Reciprocal on the special-function unit (rcp.approx: about 1 ulp; exactly 1 for 1).
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Backward of 8x8 tiles with one pixel per thread, entry-parallel gradient
 // sums, each warp on its own.  A work item is one 8x4 block of a tile (or of a
 // chunk of a split tile), taken by the warp from the shared counter; no
 // CTA-wide barrier, so the two blocks of a tile, whose lists and walks
 // differ, do not wait for each other.  The warp walks back from the largest
-// `last` of its own 32 pixels and stages, in batches of 32 candidates, only
-// the entries some pixel of its block blended (the forward's per-block bit,
-// or every flagged entry when the forward ran at another launch shape; the
-// block-rectangle alpha test when there are no flags).  Per group of 16
-// staged entries:
-//   A. pixel-parallel (lane = pixel): walks the group's entries back to front
-//      exactly as k_render_bwd (the forward's blend test bit for bit, T
-//      recovered through 1/(1 - alpha), dL/dalpha from the running g . S) and
-//      stores per (entry, pixel) the two scalars the gradient needs,
-//      dp = dL/dpower and wT = alpha T (0, 0 where the pixel does not blend).
-//      Four entries at a time: their tests, alphas and reciprocals do not
-//      depend on the transmittance chain and are formed first;
-//   B. entry-parallel (lane = entry of the group, one of two 8x2 halves of the
-//      block): the sums over the half's pixels of dp dx, dp dy, dp dx^2,
-//      dp dx dy, dp dy^2 (dx, dy: Gaussian centre minus pixel centre) follow
-//      from moments of dp about the half's centre, whose pixel offsets are
-//      compile-time constants (per row sum dp and sum dp ox, and sum dp ox^2;
-//      ox in -3.5 .. 3.5, oy = -0.5 / +0.5; expanding about the half's own
-//      centre keeps cancellation small), plus the colour sums sum wT dL/dC;
-//      one shuffle adds the halves and three vector atomics per entry go out.
+// `last` of its own 32 pixels over batches of 32 candidates and stages, last
+// entry first, only those that some pixel of its block blended (the forward's
+// per-block bit, or every flagged entry when the forward ran at another launch
+// shape; the block-rectangle alpha test when there are no flags).  The staged
+// entries form a ring that carries over from batch to batch, so every group but
+// the walk's last is full.  Per group of 16 entries:
+//   A. pixel-parallel (lane = pixel): walks the group's entries exactly as
+//      k_render_bwd (the forward's blend test bit for bit, T recovered through
+//      1/(1 - alpha), dL/dalpha from the running g . S) and stores per (entry,
+//      pixel) the two scalars the gradient needs, dp = dL/dpower and wT =
+//      alpha T.  One straight line for the whole warp, two entries a step in
+//      packed float32: where the pixel does not blend, alpha is 0, which leaves
+//      T and g . S alone and gives dp = wT = 0;
+//   B. entry-parallel (lane = entry pair of the group and one row of the block):
+//      the sums over the pixels of dp dx, dp dy, dp dx^2, dp dx dy, dp dy^2 (dx,
+//      dy: Gaussian centre minus pixel centre) follow from moments of dp about
+//      the block's centre (per row sum dp, sum dp ox, sum dp ox^2 with ox in
+//      -3.5 .. 3.5; expanding about the block's own centre keeps cancellation
+//      small), packed over the two entries, plus the colour sums sum wT dL/dC with
+//      the row's dL/dC in registers.  Two rounds of shuffles join the rows, the
+//      first also leaving one entry per lane; then two lanes hold each entry's
+//      sums and add their parts of its record.
 // The opacity term uses d alpha / d o = alpha / o below the clamp: sum(dp) / o.
+// Bound by issue and the shared-memory pipe together (77% of the issue slots,
+// 85% of the pipe's wavefronts).  Measured on 16 views of 1237x822, 480k
+// Gaussians, mixed records: 4.14 ms with groups cut at every batch (9.5 entries
+// of 16 on average) and a scalar walk with branches -> 3.55 ms (on four of the
+// views 1097M -> 740M warp instructions; then the shared-memory pipe was full)
+// -> 3.25 ms with a pair and a row per lane instead of an entry and half the
+// block -> 3.20 ms with the row's dL/dC in registers instead of read from shared
+// memory per group (12 blocks of 64 threads per SM; 9, 10, 11 blocks 3.21, 3.23,
+// 3.20 ms).
 template <int REC>
-__global__ void __launch_bounds__(64, 14)
+__global__ void __launch_bounds__(64, 12)
 k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
                 const uint2* __restrict__ ranges, RViews rv, RHdr* hdr, const int4* __restrict__ items, Slots sl,
                 const uint8_t* __restrict__ flags, long long flags_cap,
@@ -924,25 +945,23 @@ k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
                 const float* __restrict__ dLdimg, float4* __restrict__ grad2d)
 {
     constexpr int B = 8, NPIX = 64;
-    __shared__ float4 s_a[2][32];    // u, v, a', b'  (the forward's prescaled conic)
-    __shared__ float2 s_q[2][32];    // c', log2 o
-    __shared__ float4 s_k[2][32];    // A, B, C, 1/o
-    __shared__ float4 s_col[2][32];  // r, g, b, list position (int bits)
-    __shared__ uint32_t s_g[2][32];
-    __shared__ float2 s_m[2][kEpG * kEpPitch];  // per warp: [entry][pixel] (dp, wT)
-    __shared__ float4 s_gp[2][32];               // per warp: dL/dC of its pixels
+    // staged entry pairs: (u, u', v, v'), (a, a', b, b') the forward's prescaled
+    // conic, (c, c', log2 o, log2 o'), (r, r', g, g'), (b, b', list positions)
+    __shared__ float4 s_pair[2][kEpRing / 2 * kPairW];
+    __shared__ float4 s_k[2][kEpRing];           // A, B, C, 1/o
+    __shared__ uint32_t s_g[2][kEpRing];
+    __shared__ float4 s_m[2][kEpG / 2 * kEpPitch];  // [pair][pixel] (dp, dp', wT, wT')
+    __shared__ float4 s_px[2][32];               // per pixel dL/dC
     const float bg0 = rv.bg0, bg1 = rv.bg1, bg2 = rv.bg2;
     const bool planned = hdr->planned != 0 && items != nullptr;
     const int L = planned ? hdr->L : INT_MAX;
     const int count = planned ? hdr->n_items : rv.total;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    float2* sm = s_m[wp];
-    float4* wa = s_a[wp];
-    float2* wq = s_q[wp];
-    float4* wk = s_k[wp];
-    float4* wc = s_col[wp];
-    uint32_t* wg = s_g[wp];
-    const uint32_t lt = (1u << lane) - 1u;
+    float4* const sp = s_pair[wp];
+    float4* const sm = s_m[wp];
+    float4* const wk = s_k[wp];
+    uint32_t* const wg = s_g[wp];
+    const uint32_t above = ~((2u << lane) - 1u);  // lanes behind this one in the list
     for (;;) {
     int blk = 0;
     const Item it = next_item_warp(&hdr->cnt_bwd, count, planned ? items : nullptr, rv, &blk);
@@ -979,20 +998,29 @@ k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
             gS = T * (g0 * bg0 + g1 * bg1 + g2 * bg2);
         }
     }
-    s_gp[wp][lane] = make_float4(g0, g1, g2, 0.f);
+    __syncwarp();
+    s_px[wp][lane] = make_float4(g0, g1, g2, 0.f);
+    __syncwarp();
+    // phase B: dL/dC of the 8 pixels of this lane's row
+    float gpr[8], gpg[8], gpb[8];
+#pragma unroll
+    for (int px = 0; px < 8; ++px) {
+        const float4 c = s_px[wp][8 * (lane >> 3) + px];
+        gpr[px] = c.x; gpg[px] = c.y; gpb[px] = c.z;
+    }
     const int top = min(__reduce_max_sync(0xffffffffu, lastp), hi);
-    // phase B: this lane's entry of the group and half of the block's pixels
-    // (pixels 16 h .. 16 h + 15 = rows 2h, 2h + 1 of the block)
-    const int be = lane & (kEpG - 1), bh = lane >> 4;
-    const float bpx0 = bx0, bpy0 = by0 + (float)(2 * bh);
+    // phase B: this lane's entry pair of the group and row of the block; the
+    // entry it is left with after the first exchange
+    const int bp8 = lane & 7, br = lane >> 3, be = 2 * bp8 + (br & 1);
+    const float bcx = bx0 + 3.5f, bcy = by0 + 1.5f;
+    const float oyo = (float)br - 1.5f, oyp = (float)(br ^ 1) - 1.5f;  // this row's and the exchanged row's offsets
+    const f32x2 npx = f2_pack(-pxc, -pxc), npy = f2_pack(-pyc, -pyc);
+    const f32x2 gr = f2_pack(g0, g0), gg = f2_pack(g1, g1), gb2 = f2_pack(g2, g2);
     __syncwarp();
     // the flag byte and Gaussian index of a batch are loaded one batch ahead,
-    // so a batch waits only for its records (kNoFlag: no flag for the entry);
-    // 14 blocks per SM (72 registers) leave room for them (16 blocks at 64
-    // registers spilled: 0.466 -> 0.478 ms; 14 blocks without them 0.450,
-    // with them 0.435 ms, 12 blocks 0.444 ms)
+    // so a batch waits only for its records (kNoFlag: no flag for the entry)
     constexpr uint32_t kNoFlag = 0x100u;
-    const int base0 = top > lo ? lo + ((top - lo - 1) / 32) * 32 : lo - 1;
+    int base = top > lo ? lo + ((top - lo - 1) / 32) * 32 : lo - 1;
     uint32_t fn = kNoFlag, gn = 0;
     auto fetch = [&](int b) {
         const int jj = b + lane;
@@ -1004,135 +1032,171 @@ k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
             gn = gid[gj];
         }
     };
-    fetch(base0);
-    for (int base = base0; base >= lo; base -= 32) {
-        const int j = base + lane;
-        const uint32_t fcur = fn, g = gn;
-        fetch(base - 32);
-        bool keep = false;
-        float4 ga, gb;
-        float gc = 0.f;
-        if (j < top) {
-            if (fcur != kNoFlag) {
-                keep = (fcur & kFlagWarpBits) ? ((fcur >> blk) & 1u) != 0 : fcur != 0;
-                if (keep) load_record<REC>(feat, g, ga, gb, gc);
-            } else {
-                load_record<REC>(feat, g, ga, gb, gc);
-                keep = !tile_skip(ga, gb, bx0, bx1, by0, by1);
+    fetch(base);
+    int pend = 0, gslot = 0;  // staged entries, and the ring slot of the first
+    for (;;) {
+        while (pend < kEpG && base >= lo) {
+            const int j = base + lane;
+            const uint32_t fcur = fn, g = gn;
+            base -= 32;
+            fetch(base);
+            bool keep = false;
+            float4 ga, gb;
+            float gc = 0.f, lo2 = 0.f;
+            if (j < top) {
+                if (fcur != kNoFlag) {
+                    keep = (fcur & kFlagWarpBits) ? ((fcur >> blk) & 1u) != 0 : fcur != 0;
+                    if (keep) {
+                        load_record<REC>(feat, g, ga, gb, gc);
+                        lo2 = __log2f(gb.y);
+                    }
+                } else {
+                    load_record<REC>(feat, g, ga, gb, gc);
+                    lo2 = __log2f(gb.y);
+                    keep = !block_skip(ga, gb, lo2, bx0, bx1, by0, by1);
+                }
             }
+            const uint32_t km = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                int slot = gslot + pend + __popc(km & above);
+                if (slot >= kEpRing) slot -= kEpRing;
+                float4* q = sp + (slot >> 1) * kPairW;
+                float* f = (float*)q + (slot & 1);
+                f[0] = ga.x; f[2] = ga.y;
+                f[4] = -0.5f * kLog2e * ga.z; f[6] = -kLog2e * ga.w;
+                f[8] = -0.5f * kLog2e * gb.x; f[10] = lo2;
+                f[12] = gb.z; f[14] = gb.w;
+                f[16] = gc; f[18] = __int_as_float(j);
+                wg[slot] = g;
+                wk[slot] = make_float4(ga.z, ga.w, gb.x, __frcp_rn(gb.y));
+            }
+            pend += __popc(km);
         }
-        const uint32_t km = __ballot_sync(0xffffffffu, keep);
-        const int cnt = __popc(km);
-        if (keep) {
-            const int slot = __popc(km & lt);
-            wg[slot] = g;
-            wa[slot] = make_float4(ga.x, ga.y, -0.5f * kLog2e * ga.z, -kLog2e * ga.w);
-            wq[slot] = make_float2(-0.5f * kLog2e * gb.x, __log2f(gb.y));
-            wk[slot] = make_float4(ga.z, ga.w, gb.x, __frcp_rn(gb.y));
-            wc[slot] = make_float4(gb.z, gb.w, gc, __int_as_float(j));
+        if (pend == 0) break;
+        const int n = min(pend, kEpG);
+        if ((n & 1) && lane == 0) {  // (only the walk's last group) an entry no pixel blends
+            float* f = (float*)(sp + ((gslot + n) >> 1) * kPairW) + 1;
+#pragma unroll
+            for (int i = 0; i < 18; i += 2) f[i] = 0.f;
+            f[18] = __int_as_float(INT_MAX);
         }
         __syncwarp();
-        for (int kb = ((cnt - 1) / kEpG) * kEpG; kb >= 0 && cnt > 0; kb -= kEpG) {
-            const int ke = min(cnt, kb + kEpG);
-            // A: this lane's pixel over the group's entries, back to front, four at a time
-            uint32_t mine = 0;
-            for (int k0 = ke - 1; k0 >= kb; k0 -= 4) {
-                float al[4], iv[4], gcl[4];
-                bool bl[4], un[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int kk = k0 - u >= kb ? k0 - u : kb;
-                    const float4 col = wc[kk];
-                    const float4 a = wa[kk];
-                    const float2 q = wq[kk];
-                    const float dx = a.x - pxc, dy = a.y - pyc;
-                    const float p = fmaf(dx, fmaf(a.w, dy, a.z * dx), q.x * dy * dy);
-                    const float e = p + q.y;
-                    bl[u] = k0 - u >= kb && __float_as_int(col.w) < lastp && p <= 0.f && e >= kLog2AlphaMin;
-                    const float raw = ex2_approx(e);
-                    al[u] = fminf(kAlphaMax, raw);
-                    un[u] = raw <= kAlphaMax;
-                    iv[u] = __fdividef(1.f, 1.f - al[u]);
-                    gcl[u] = fmaf(g0, col.x, fmaf(g1, col.y, g2 * col.z));
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (k0 - u < kb) break;
-                    float dpv = 0.f, wTv = 0.f;
-                    if (bl[u]) {
-                        T *= iv[u];
-                        wTv = al[u] * T;
-                        const float dLda = fmaf(T, gcl[u], -gS * iv[u]);
-                        gS = fmaf(wTv, gcl[u], gS);
-                        dpv = un[u] ? dLda * al[u] : 0.f;
-                        mine |= 1u << (k0 - u - kb);
-                    }
-                    sm[(k0 - u - kb) * kEpPitch + lane] = make_float2(dpv, wTv);
-                }
+        // A: this lane's pixel over the group's entries, back to front, two at a time
+        uint32_t mine = 0;
+        {
+            const float4* q = sp + (gslot >> 1) * kPairW;
+            float4* out = sm + lane;
+            uint32_t bit = 1u;
+            for (int k = 0; k < n; k += 2, q += kPairW, out += kEpPitch, bit <<= 2) {
+                const float4 uv = q[0], ab = q[1], cl = q[2], rgc = q[3], bp = q[4];
+                const f32x2 dx = f2_add(f2_pack(uv.x, uv.y), npx), dy = f2_add(f2_pack(uv.z, uv.w), npy);
+                const f32x2 pu = f2_fma(dx, f2_fma(f2_pack(ab.z, ab.w), dy, f2_mul(f2_pack(ab.x, ab.y), dx)),
+                                        f2_mul(f2_mul(f2_pack(cl.x, cl.y), dy), dy));
+                const f32x2 eu = f2_add(pu, f2_pack(cl.z, cl.w));
+                const f32x2 gu = f2_fma(gr, f2_pack(rgc.x, rgc.y),
+                                        f2_fma(gg, f2_pack(rgc.z, rgc.w), f2_mul(gb2, f2_pack(bp.x, bp.y))));
+                float p0, p1, e0, e1, gc0, gc1;
+                f2_unpack(pu, p0, p1);
+                f2_unpack(eu, e0, e1);
+                f2_unpack(gu, gc0, gc1);
+                const bool b0 = __float_as_int(bp.z) < lastp && p0 <= 0.f && e0 >= kLog2AlphaMin;
+                const bool b1 = __float_as_int(bp.w) < lastp && p1 <= 0.f && e1 >= kLog2AlphaMin;
+                const float r0 = ex2_approx(e0), r1 = ex2_approx(e1);
+                const float a0 = b0 ? fminf(kAlphaMax, r0) : 0.f, a1 = b1 ? fminf(kAlphaMax, r1) : 0.f;
+                const float i0 = rcp_approx(1.f - a0), i1 = rcp_approx(1.f - a1);
+                // transmittance in front of the entry, then dL/dalpha and the colour behind the next
+                T *= i0;
+                const float w0 = a0 * T;
+                const float d0 = fmaf(T, gc0, -gS * i0);
+                gS = fmaf(w0, gc0, gS);
+                T *= i1;
+                const float w1 = a1 * T;
+                const float d1 = fmaf(T, gc1, -gS * i1);
+                gS = fmaf(w1, gc1, gS);
+                // below the clamp d alpha / d power = alpha
+                const float dp0 = b0 && r0 <= kAlphaMax ? d0 * a0 : 0.f;
+                const float dp1 = b1 && r1 <= kAlphaMax ? d1 * a1 : 0.f;
+                if (b0) mine |= bit;
+                if (b1) mine |= bit << 1;
+                *out = make_float4(dp0, dp1, w0, w1);
             }
-            const uint32_t used = __reduce_or_sync(0xffffffffu, mine);
-            __syncwarp();
-            if (used) {
-                const int ek = kb + be;
-                const bool act = ek < ke && ((used >> be) & 1u);
-                float4 kc = make_float4(0.f, 0.f, 0.f, 0.f);
-                float dx0 = 0.f, dy0 = 0.f;
-                if (act) {
-                    kc = wk[ek];
-                    const float4 a = wa[ek];
-                    dx0 = a.x - (bpx0 + 3.5f);
-                    dy0 = a.y - (bpy0 + 0.5f);
-                }
-                float s0a = 0.f, s0b = 0.f, sxa = 0.f, sxb = 0.f, sxx = 0.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-                const float2* row = sm + be * kEpPitch + 16 * bh;
-                const float4* gpx = s_gp[wp] + 16 * bh;
-#pragma unroll 1
-                for (int r = 0; r < 2; ++r) {
-                    float s0 = 0.f, sx = 0.f;
-#pragma unroll
-                    for (int px = 0; px < 8; ++px) {
-                        const float2 m = row[8 * r + px];
-                        const float4 gp = gpx[8 * r + px];
-                        const float ox = (float)px - 3.5f;
-                        s0 += m.x;
-                        sx = fmaf(m.x, ox, sx);
-                        sxx = fmaf(m.x, ox * ox, sxx);
-                        c0 = fmaf(m.y, gp.x, c0);
-                        c1 = fmaf(m.y, gp.y, c1);
-                        c2 = fmaf(m.y, gp.z, c2);
-                    }
-                    if (r == 0) { s0a = s0; sxa = sx; } else { s0b = s0; sxb = sx; }
-                }
-                const float S0 = s0a + s0b, Sx = sxa + sxb, Sy = 0.5f * (s0b - s0a), Sxy = 0.5f * (sxb - sxa);
-                const float Syy = 0.25f * S0;
-                const float qx = fmaf(dx0, S0, -Sx), qy = fmaf(dy0, S0, -Sy);
-                float acc[9];
-                acc[0] = fmaf(kc.x, qx, kc.y * qy);
-                acc[1] = fmaf(kc.y, qx, kc.z * qy);
-                acc[2] = fmaf(dx0, fmaf(dx0, S0, -2.f * Sx), sxx);
-                acc[3] = fmaf(dx0, fmaf(dy0, S0, -Sy), fmaf(-dy0, Sx, Sxy));
-                acc[4] = fmaf(dy0, fmaf(dy0, S0, -2.f * Sy), Syy);
-                acc[5] = S0;
-                acc[6] = c0;
-                acc[7] = c1;
-                acc[8] = c2;
-#pragma unroll
-                for (int i = 0; i < 9; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
-                if (act && bh == 0) {
-                    float4* gq = grad2d + 3 * (size_t)wg[ek];
-                    atomicAdd(gq, make_float4(-acc[0], -acc[1], -0.5f * acc[2], -acc[3]));
-                    atomicAdd(gq + 1, make_float4(-0.5f * acc[4], acc[5] * kc.w, acc[6], acc[7]));
-                    atomicAdd((float*)(gq + 2), acc[8]);
-                }
-            }
-            __syncwarp();
         }
+        const uint32_t used = __reduce_or_sync(0xffffffffu, mine);
+        __syncwarp();
+        if (used) {
+            // (slots of a partial group hold an earlier group's entries: their sums are not used)
+            const float4* const row = sm + bp8 * kEpPitch + 8 * br;
+            // (both entries at once) sum dp, sum dp ox, sum dp ox^2: ox = -3.5 .. 3.5, so
+            // pixels px and 7 - px share their sum and difference
+            f32x2 s0, sx, sxx;
+            float c0[3], c1[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) c0[i] = c1[i] = 0.f;
+#pragma unroll
+            for (int px = 0; px < 4; ++px) {
+                const float4 m = row[7 - px], n2 = row[px];
+                const float k = 3.5f - (float)px;
+                const f32x2 d = f2_pack(m.x, m.y), e = f2_pack(n2.x, n2.y);
+                const f32x2 su = f2_add(d, e), di = f2_fma(e, f2_pack(-1.f, -1.f), d);
+                s0 = px ? f2_add(s0, su) : su;
+                sx = px ? f2_fma(di, f2_pack(k, k), sx) : f2_mul(di, f2_pack(k, k));
+                sxx = px ? f2_fma(su, f2_pack(k * k, k * k), sxx) : f2_mul(su, f2_pack(k * k, k * k));
+                c0[0] = fmaf(m.z, gpr[7 - px], fmaf(n2.z, gpr[px], c0[0]));
+                c0[1] = fmaf(m.z, gpg[7 - px], fmaf(n2.z, gpg[px], c0[1]));
+                c0[2] = fmaf(m.z, gpb[7 - px], fmaf(n2.z, gpb[px], c0[2]));
+                c1[0] = fmaf(m.w, gpr[7 - px], fmaf(n2.w, gpr[px], c1[0]));
+                c1[1] = fmaf(m.w, gpg[7 - px], fmaf(n2.w, gpg[px], c1[1]));
+                c1[2] = fmaf(m.w, gpb[7 - px], fmaf(n2.w, gpb[px], c1[2]));
+            }
+            // even rows keep the pair's first entry, odd rows the second
+            float va[6], vb[6];
+            f2_unpack(s0, va[0], vb[0]); f2_unpack(sx, va[1], vb[1]); f2_unpack(sxx, va[2], vb[2]);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) { va[3 + i] = c0[i]; vb[3 + i] = c1[i]; }
+            const bool odd = (br & 1) != 0;
+            float acc[9];  // S0, Sx, Sxx, red, green, blue, Sy, Sxy, Syy
+            {
+                float own[6], oth[6];
+#pragma unroll
+                for (int i = 0; i < 6; ++i) {
+                    own[i] = odd ? vb[i] : va[i];
+                    oth[i] = __shfl_xor_sync(0xffffffffu, odd ? va[i] : vb[i], 8);
+                    acc[i] = own[i] + oth[i];
+                }
+                const float yo = oyo * own[0], yp = oyp * oth[0];
+                acc[6] = yo + yp;
+                acc[7] = fmaf(oyo, own[1], oyp * oth[1]);
+                acc[8] = fmaf(oyo, yo, oyp * yp);
+            }
+#pragma unroll
+            for (int i = 0; i < 9; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+            if ((used >> be) & 1u) {
+                const int slot = gslot + be;
+                const float4 kc = wk[slot];
+                const float* f = (const float*)(sp + (slot >> 1) * kPairW) + (slot & 1);
+                const float dx0 = f[0] - bcx, dy0 = f[2] - bcy;
+                const float S0 = acc[0], Sx = acc[1], Sy = acc[6];
+                float4* const gq = grad2d + 3 * (size_t)wg[slot];
+                if (br < 2) {
+                    const float qx = fmaf(dx0, S0, -Sx), qy = fmaf(dy0, S0, -Sy);
+                    const float gA = fmaf(dx0, fmaf(dx0, S0, -2.f * Sx), acc[2]);
+                    const float gB = fmaf(dx0, fmaf(dy0, S0, -Sy), fmaf(-dy0, Sx, acc[7]));
+                    atomicAdd(gq, make_float4(-fmaf(kc.x, qx, kc.y * qy), -fmaf(kc.y, qx, kc.z * qy), -0.5f * gA, -gB));
+                } else {
+                    const float gC = fmaf(dy0, fmaf(dy0, S0, -2.f * Sy), acc[8]);
+                    atomicAdd(gq + 1, make_float4(-0.5f * gC, S0 * kc.w, acc[3], acc[4]));
+                    atomicAdd((float*)(gq + 2), acc[5]);
+                }
+            }
+        }
+        __syncwarp();
+        pend -= n;
+        gslot += kEpG;
+        if (gslot == kEpRing) gslot = 0;
     }
     __syncwarp();
     }  // work items
 }
-
-constexpr int kPairW = 5;                     // float4 per staged entry pair
 
 // Forward of 8x8 tiles with one pixel per thread, each warp on its own: a work
 // item is one 8x4 block of a tile (or of a chunk of a split tile), taken per
