@@ -183,8 +183,9 @@ static TileKey tile_key(const TileGrid& tg)
     return k;
 }
 
-// A record in depth order: rect corner x0 | y0 << 16, tile mask (or, with the
-// top bit of .w set, the rect's width and height), and its index in the view.
+// A record in depth order: rect corner x0 | y0 << 16, tile mask (of a whole rect
+// too, up to 8 x 8 tiles; with the top bit of .w set, a larger rect's width and
+// height), and its index in the view.
 constexpr uint32_t kRectFlag = 0x80000000u;
 
 // One tile of REC_TILE records of a view in depth order: gathers each one's
@@ -260,8 +261,13 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
 #pragma unroll
     for (int k = 0; k < REC_IPT; ++k) {
         const Rect q = tile_rect(uv[k].x, uv[k].y, rad[k], B, TX, TY);
-        const uint32_t mlo = __float_as_uint(f2[k].y), mhi = __float_as_uint(f2[k].z);
+        uint32_t mlo = __float_as_uint(f2[k].y), mhi = __float_as_uint(f2[k].z);
         const uint32_t w = (uint32_t)(q.x1 - q.x0), h = (uint32_t)(q.y1 - q.y0);
+        if ((mlo | mhi) == 0 && w <= 8 && h <= 8) {  // a whole rect that fits a mask
+            const uint32_t rows = 0x01010101u * ((1u << w) - 1u);
+            mlo = h >= 4 ? rows : rows & ((1u << (8 * h)) - 1u);
+            mhi = h <= 4 ? 0u : h == 8 ? rows : rows & ((1u << (8 * (h - 4))) - 1u);
+        }
         const bool masked = (mlo | mhi) != 0;
         out[k] = make_uint4((uint32_t)q.x0 | ((uint32_t)q.y0 << 16), masked ? mlo : w, masked ? mhi : h,
                             (uint32_t)(r[k] - (uint32_t)(st.v * P)) | (masked ? 0u : kRectFlag));
@@ -370,8 +376,9 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
 // First tile pass: the pairs of its tile, formed from the records in depth
 // order.  A thread takes a record and writes its pairs to their places in
 // shared memory (tile mask: a walk over the set bits, at most 64); the rects
-// without a mask, of any size, are written by the whole warp, 32 pairs at a
-// time.  (One thread per 16 consecutive pairs, walking along the records, left
+// larger than a mask are written by the whole warp, 32 pairs at a time (small
+// whole rects too took the pass 280 instead of 40 us on 1.6M records of one or
+// two tiles).  (One thread per 16 consecutive pairs, walking along the records, left
 // 16-way bank conflicts and a chain of dependent record loads.  A warp-round
 // of 32 records takes about 240 instructions; issue and the pass behind it bound
 // the kernel: 96 us on 5.9M pairs.)
