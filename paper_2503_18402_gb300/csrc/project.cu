@@ -465,18 +465,42 @@ k_project_bwd(float* __restrict__ prm, long long stride, int P, ViewSet vs_host,
     #pragma unroll
         for (int k = 0; k < (SINGLE ? 1 : NB); ++k) dsh[k][0] = dsh[k][1] = dsh[k][2] = 0.f;
         bool any = false;
-        for (int v = 0; v < vs.n; ++v) {
-            const size_t r = (size_t)v * P + i;
-            if (radius[r] == 0) continue;
+        // the views that see the Gaussian (all radii loaded at once); a view's 2D
+        // gradients are loaded while the view before it is worked on, so a view
+        // waits for memory only when nothing was left to do meanwhile (SINGLE: one view)
+        uint32_t seen = 0;
+        if (SINGLE) {
+            seen = radius[i] != 0 ? 1u : 0u;
+        } else {
+#pragma unroll
+            for (int v = 0; v < DG_MAX_VIEWS; ++v)
+                if (v < vs.n) seen |= (radius[(size_t)v * P + i] != 0 ? 1u : 0u) << v;
+        }
+        float4 n0, n1;
+        float n2 = 0.f;
+        uint8_t ncm = 0;
+        auto fetch = [&](uint32_t left) {
+            if (!left) return;
+            const size_t r = (size_t)(__ffs((int)left) - 1) * P + i;
+            n0 = grad2d[3 * r];
+            n1 = grad2d[3 * r + 1];
+            n2 = grad2d[3 * r + 2].x;
+            ncm = clampm[r];
+        };
+        fetch(seen);
+        for (; seen; seen &= seen - 1) {
+            const int v = SINGLE ? 0 : __ffs((int)seen) - 1;
+            const float4 g0 = n0, g1 = n1;
+            const float g2x = n2;
+            const uint8_t cm = ncm;
+            if (!SINGLE) fetch(seen & (seen - 1));
             const Cam& cam = vs.cam[v];
             Splat S;
             if (!splat(g, cam, near_plane, eps2d, mip2d, S)) continue;
             any = true;
-            const float4 g0 = grad2d[3 * r], g1 = grad2d[3 * r + 1], g2 = grad2d[3 * r + 2];
             const float dLu = g0.x, dLv = g0.y, dLA = g0.z, dLB = g0.w, dLC = g1.x;
             dop += g1.y * S.comp;  // record opacity = sigmoid * comp
-            const uint8_t cm = clampm[r];
-            const float dcol[3] = {(cm & 1u) ? 0.f : g1.z, (cm & 2u) ? 0.f : g1.w, (cm & 4u) ? 0.f : g2.x};
+            const float dcol[3] = {(cm & 1u) ? 0.f : g1.z, (cm & 2u) ? 0.f : g1.w, (cm & 4u) ? 0.f : g2x};
             // colour: SH coefficients and the view direction
             {
                 float d0 = g.p[0] - vs.campos[v][0], d1 = g.p[1] - vs.campos[v][1], d2 = g.p[2] - vs.campos[v][2];

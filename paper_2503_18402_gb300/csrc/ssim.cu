@@ -449,7 +449,7 @@ k_ssim_bwd(const float* __restrict__ img, const float* __restrict__ tgt, SViews 
 }  // namespace dg
 
 // Rows of a segment: the longest of 64, 32, 16 that gives at least five blocks
-// per SM, else 16: a segment repeats the window sums of ten rows.  (16 views of
+// per SM, else 8: a segment repeats the window sums of ten rows.  (16 views of
 // 1237x822: 64 rows 0.615 ms, 128 0.635; one view, in a training step: 32 rows 8 us
 // less than 16.)
 static bool ssim_views(const int32_t* wh, int n_views, dg::SViews* sv, long long* nmap)
@@ -479,7 +479,7 @@ static bool ssim_views(const int32_t* wh, int n_views, dg::SViews* sv, long long
         }
         sv->boff[n_views] = (int)blocks;
         *nmap = map;
-        if (blocks >= 5 * 152 || rows == 16) return true;
+        if (blocks >= 5 * 152 || rows == 8) return true;
     }
 }
 
@@ -489,7 +489,7 @@ static size_t ssim_map_bytes(long long nmap) { return ((size_t)3 * nmap * sizeof
 static size_t ssim_ws_bytes(const dg::SViews& sv, long long nmap)
 {
     size_t blocks = 0;
-    for (int v = 0; v < sv.n; ++v) blocks += (size_t)3 * sv.TX[v] * ((sv.H[v] + 15) / 16);
+    for (int v = 0; v < sv.n; ++v) blocks += (size_t)3 * sv.TX[v] * ((sv.H[v] + 7) / 8);
     return 16 + ssim_map_bytes(nmap) + sizeof(float2) * blocks;
 }
 
