@@ -449,7 +449,9 @@ DG_API dg_status dg_densify_mark(const float* params, int64_t stride, int64_t P,
  * Gaussians to dst (planar [59][dst_stride], dst_stride >= P + min(n_cand,
  * budget)) and their Adam moments; noise [min(n_cand,budget)][2][3] standard
  * normals for the j-th selected Gaussian (index order); *P_out (device int64)
- * = N' + number selected.  Sources and destinations must not overlap. */
+ * = N' + number selected (or DG_ERR_TIMEOUT when a bounded wait between thread
+ * blocks gave up, which does not happen when the device runs the launch to
+ * completion; nothing is written then).  Sources and destinations must not overlap. */
 DG_API dg_status dg_densify_apply(const float* params, const float* m, const float* v, int64_t stride, int64_t P,
                                   int64_t n_cand, int64_t budget, const float* noise, void* ws, size_t ws_bytes,
                                   float* dst_params, float* dst_m, float* dst_v, int64_t dst_stride,

@@ -37,7 +37,7 @@
 // most two of them per SM.
 #pragma once
 
-#include "radix.cuh"
+#include "scan.cuh"
 
 namespace dg {
 namespace {

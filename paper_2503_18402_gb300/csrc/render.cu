@@ -57,7 +57,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
-#include "radix.cuh"
+#include "scan.cuh"
 
 namespace dg {
 
