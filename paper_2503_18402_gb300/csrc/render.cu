@@ -270,6 +270,74 @@ __global__ void k_plan_items(const uint2* __restrict__ ranges, int n_tiles, RHdr
     }
 }
 
+// The whole plan in one block, for up to PLAN_TILES tiles: every automatic split
+// of 8x8 tiles (it happens below two tiles per resident CTA, 4864 here) and of
+// 16x16 tiles of common images.  A plan of a few tiles is launch-bound: the six
+// scan launches took 33 us from the first's start to the last's end at 16 tiles,
+// this one takes 5 us; 1k Gaussians at 64x64, forward and backward through the
+// autograd call: 513 -> 467 us.  Above it the scan's blocks read the ranges in parallel.
+constexpr int PLAN_THREADS = 1024;
+constexpr int PLAN_IPT = 8;
+constexpr int PLAN_TILES = PLAN_THREADS * PLAN_IPT;
+__global__ void __launch_bounds__(PLAN_THREADS)
+k_plan_small(const uint2* __restrict__ ranges, int n_tiles, RHdr* hdr, SplitCfg cfg, int4* __restrict__ items,
+             int4* __restrict__ sitems)
+{
+    __shared__ uint64_t sm[33];
+    const int lane = threadIdx.x & 31;
+    const int t0 = threadIdx.x * PLAN_IPT;
+    long long len[PLAN_IPT];
+    uint64_t acc = 0, tot;
+#pragma unroll
+    for (int i = 0; i < PLAN_IPT; ++i) {
+        len[i] = 0;
+        if (t0 + i < n_tiles) {
+            const uint2 r = ranges[t0 + i];
+            len[i] = (long long)(r.y - r.x);
+        }
+        acc += (uint64_t)len[i];
+    }
+    block_excl_scan<uint64_t>(acc, sm, &tot);
+    const long long M = (long long)tot;
+    const int L = split_len(M, cfg);
+    // items (low 32 bits) and split chunks (high 32 bits) of the thread's tiles
+    int k[PLAN_IPT];
+    uint64_t cnt = 0;
+#pragma unroll
+    for (int i = 0; i < PLAN_IPT; ++i) {
+        k[i] = t0 + i >= n_tiles ? 0 : len[i] <= L ? 1 : (int)((len[i] + L - 1) / L);
+        cnt += (uint64_t)k[i] | (k[i] > 1 ? (uint64_t)k[i] << 32 : 0);
+    }
+    uint64_t off = block_excl_scan<uint64_t>(cnt, sm, &tot);
+    if (threadIdx.x == 0) {
+        hdr->M = M;
+        hdr->totals = (long long)tot;
+        hdr->L = L;
+        hdr->n_items = (int)(tot & 0xffffffffull);
+        hdr->n_slots = (int)(tot >> 32);
+        hdr->planned = 1;
+    }
+#pragma unroll
+    for (int i = 0; i < PLAN_IPT; ++i) {
+        const int io = (int)(off & 0xffffffffull), so = (int)(off >> 32);
+        if (k[i] == 1) items[io] = make_int4(t0 + i, 0, 1, -1);
+        // a split tile's chunks are written by the whole warp
+        uint32_t todo = __ballot_sync(0xffffffffu, k[i] > 1);
+        while (todo) {
+            const int l = __ffs((int)todo) - 1;
+            todo &= todo - 1;
+            const int kk = __shfl_sync(0xffffffffu, k[i], l), it = __shfl_sync(0xffffffffu, t0 + i, l);
+            const int io_l = __shfl_sync(0xffffffffu, io, l), so_l = __shfl_sync(0xffffffffu, so, l);
+            for (int c = lane; c < kk; c += 32) {
+                const int4 w = make_int4(it, c, kk, so_l);
+                items[io_l + c] = w;
+                sitems[so_l + c] = w;
+            }
+        }
+        off += (uint64_t)k[i] | (k[i] > 1 ? (uint64_t)k[i] << 32 : 0);
+    }
+}
+
 // A work item: tile (global over views), chunk c of nch, first chunk slot
 // (-1: the tile is not split), and the tile's place in its view.
 struct Item { int tile, c, nch, slot0, v, tx, ty, W, H; long long poff; };
@@ -1496,6 +1564,24 @@ static RenderWs render_ws_fixed(void* base, long long n_tiles, int B, bool split
     return w;
 }
 
+// Split plan of n tiles: hdr and the item arrays.
+static void plan_items(const uint2* rg, int n, const RenderWs& w, const dg::SplitCfg& cfg, cudaStream_t s)
+{
+    if (n <= dg::PLAN_TILES) {
+        dg::k_plan_small<<<1, dg::PLAN_THREADS, 0, s>>>(rg, n, w.hdr, cfg, w.items, w.sitems);
+        dg_note_launch();
+        return;
+    }
+    const int nb = (int)(((long long)n + dg::SCAN_TILE - 1) / dg::SCAN_TILE);
+    dg::k_scan_reduce<<<nb, dg::SCAN_THREADS, 0, s>>>(dg::LoadLen{rg}, n, w.bsum);
+    dg::k_scan_top<<<1, 1024, 0, s>>>(w.bsum, nb, &w.hdr->M);
+    dg_note_launch(2);
+    dg::exclusive_scan(dg::LoadChunks{rg, w.hdr, cfg}, n, w.toff, w.bsum, &w.hdr->totals, s);
+    const int pg = (n + 255) / 256;
+    dg::k_plan_items<<<pg < 1024 ? pg : 1024, 256, 0, s>>>(rg, n, w.hdr, cfg, w.toff, w.items, w.sitems);
+    dg_note_launch();
+}
+
 // Tile 8, one pixel per thread: the warp-per-block forward (k_render_fwd_w).
 template <int REC>
 static dg_status launch_fwd_w(const float* feat, const uint32_t* gid, const uint32_t* ranges, const dg::RViews& rv,
@@ -1510,18 +1596,11 @@ static dg_status launch_fwd_w(const float* feat, const uint32_t* gid, const uint
     const bool split = rv.total > 0 && (split_req > 0 || (split_req == 0 && rv.total < 2LL * R));
     if (split) {
         const dg::SplitCfg cfg{split_req, R, w.cap};
-        const long long n = rv.total;
-        const int nb = (int)((n + dg::SCAN_TILE - 1) / dg::SCAN_TILE);
-        dg::k_scan_reduce<<<nb, dg::SCAN_THREADS, 0, s>>>(dg::LoadLen{rg}, n, w.bsum);
-        dg::k_scan_top<<<1, 1024, 0, s>>>(w.bsum, nb, &w.hdr->M);
-        dg_note_launch(2);
-        dg::exclusive_scan(dg::LoadChunks{rg, w.hdr, cfg}, n, w.toff, w.bsum, &w.hdr->totals, s);
-        const int pg = (int)((n + 255) / 256);
-        dg::k_plan_items<<<pg < 1024 ? pg : 1024, 256, 0, s>>>(rg, (int)n, w.hdr, cfg, w.toff, w.items, w.sitems);
+        plan_items(rg, rv.total, w, cfg, s);
         auto kprod = dg::k_render_fwd_w<true, REC>;
         kprod<<<resident_ctas(kprod, 64), 64, 0, s>>>((const void*)feat, gid, rg, rv, w.hdr, w.items, w.sitems, w.sl,
                                                       nullptr, 0, img, T, last, ex, bl);
-        dg_note_launch(2);
+        dg_note_launch();
     }
     const int grid = split ? R : (R < rv.total ? R : (rv.total > 0 ? rv.total : 1));
     kern<<<grid, 64, 0, s>>>((const void*)feat, gid, rg, rv, w.hdr, w.items, w.sitems, w.sl, w.flags, w.flags_cap,
@@ -1554,18 +1633,11 @@ static dg_status launch_fwd(const float* feat, const uint32_t* gid, const uint32
     const bool split = rv.total > 0 && (split_req > 0 || (split_req == 0 && rv.total < 2LL * R));
     if (split) {
         const dg::SplitCfg cfg{split_req, R, w.cap};
-        const long long n = rv.total;
-        const int nb = (int)((n + dg::SCAN_TILE - 1) / dg::SCAN_TILE);
-        dg::k_scan_reduce<<<nb, dg::SCAN_THREADS, 0, s>>>(dg::LoadLen{rg}, n, w.bsum);
-        dg::k_scan_top<<<1, 1024, 0, s>>>(w.bsum, nb, &w.hdr->M);
-        dg_note_launch(2);
-        dg::exclusive_scan(dg::LoadChunks{rg, w.hdr, cfg}, n, w.toff, w.bsum, &w.hdr->totals, s);
-        const int pg = (int)((n + 255) / 256);
-        dg::k_plan_items<<<pg < 1024 ? pg : 1024, 256, 0, s>>>(rg, (int)n, w.hdr, cfg, w.toff, w.items, w.sitems);
+        plan_items(rg, rv.total, w, cfg, s);
         auto kprod = dg::k_render_fwd<B, PPT, true, REC>;
         kprod<<<resident_ctas(kprod, B * B / PPT), B * B / PPT, 0, s>>>(
             (const void*)feat, gid, rg, rv, w.hdr, w.items, w.sitems, w.sl, nullptr, 0, img, T, last, ex, bl);
-        dg_note_launch(2);
+        dg_note_launch();
     }
     const int grid = split ? R : (R < rv.total ? R : (rv.total > 0 ? rv.total : 1));
     kern<<<grid, B * B / PPT, 0, s>>>((const void*)feat, gid, rg, rv, w.hdr, w.items, w.sitems, w.sl, w.flags,
