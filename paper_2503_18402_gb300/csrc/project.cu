@@ -137,8 +137,7 @@ __device__ inline bool splat(const G3& g, const Cam& cam, float near_plane, floa
     S.t[2] = cam.r[6] * g.p[0] + cam.r[7] * g.p[1] + cam.r[8] * g.p[2] + cam.t[2];
     if (!(S.t[2] > near_plane)) return false;
     const float tz = S.t[2];
-    const float limx = kFrustumGuard * 0.5f * (float)cam.w / cam.fx;
-    const float limy = kFrustumGuard * 0.5f * (float)cam.h / cam.fy;
+    const float limx = cam.limx, limy = cam.limy;
     const float txtz = S.t[0] / tz, tytz = S.t[1] / tz;
     S.gx = txtz < -limx || txtz > limx;
     S.gy = tytz < -limy || tytz > limy;
@@ -204,6 +203,7 @@ __device__ inline const ViewSet& block_views(const ViewSet& vs, const dg_camera*
         s_vs->cam[v] = make_cam(cdev[v]);
         s_vs->cam[v].w = vs.cam[v].w;
         s_vs->cam[v].h = vs.cam[v].h;
+        set_guard(s_vs->cam[v]);
         cam_centre(s_vs->cam[v], s_vs->campos[v]);
         s_vs->TX[v] = vs.TX[v];
         s_vs->TY[v] = vs.TY[v];
