@@ -196,7 +196,7 @@ DG_API dg_status dg_bin_count(const float* depth, const int32_t* tiles, int64_t 
  *      ranges [2 * total tiles] uint32, [start, end) of each tile's list;
  *      status (device int32): 0, or DG_ERR_CAPACITY when M > M_cap, in which
  *              case gid is untouched and every range is empty, or
- *              DG_ERR_TIMEOUT when a bounded wait between thread blocks of
+ *              DG_ERR_TIMEOUT when a bounded wait between thread blocks
  *              gave up (lists not valid; does not happen when the device
  *              runs the launch to completion), or DG_ERR_CUDA when the records'
  *              pairs are not those counted in phase 1 (every range is empty).

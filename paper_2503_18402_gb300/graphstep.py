@@ -110,7 +110,7 @@ class StepGraph:
 
     def _copy_targets(self, targets) -> None:
         """The targets, one after another, into the graph's buffer.  Float32 images
-        on the device go in one launch (16 views of 309x205: 6 instead of 65 us,
+        on the device go in one launch (16 views of 309x205: 10 instead of 65 us,
         which sixteen copies took, half of it between them); others are copied
         (and converted) one by one, as is a single image."""
         dst = self.target
