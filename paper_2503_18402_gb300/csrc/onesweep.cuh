@@ -38,6 +38,7 @@
 #pragma once
 
 #include "scan.cuh"
+#include "tilekey.cuh"
 
 namespace dg {
 namespace {
@@ -208,7 +209,7 @@ struct OsPass {
     uint32_t* kout;        // nullable: values only
     uint32_t* vout;
     uint2* ranges;         // nullable: the last tile pass's ranges (complement of the start, end), zero before the launch
-    int xbits;             // with ranges: a key is tile row << xbits | tile column
+    int linear, xbits;     // with ranges: the form of the keys (TileKey)
     int TX[DG_MAX_VIEWS], toff[DG_MAX_VIEWS + 1];  // with ranges: tiles per row and first tile of each view
     const unsigned long long* m_views;  // nullable: the views' pair counts, summed into *m_ws and *m_out
     long long* m_ws;
@@ -447,7 +448,7 @@ k_os_pass(Src src, Segs sg, OsPass ps)
             uint32_t e = j1;
             if (sk[j1 - 1] != kk)
                 for (e = j + 1; sk[e] == kk; ++e) {}
-            const uint32_t tile = (kk >> ps.xbits) * TX + (kk & ((1u << ps.xbits) - 1u));
+            const uint32_t tile = key_tile(kk, ps.linear, ps.xbits, TX);
             if (tile < nt) {
                 atomicMax(&rg[tile].x, ~(g + j));
                 atomicMax(&rg[tile].y, g + e);

@@ -29,16 +29,9 @@
 // along, the pairs emitted to memory and histogram, scan and scatter kernels per
 // tile pass.
 #include "onesweep.cuh"
+#include "tilekey.cuh"
 
 namespace dg {
-
-struct TileGrid {
-    int n;
-    int TX[DG_MAX_VIEWS], TY[DG_MAX_VIEWS];
-    int off[DG_MAX_VIEWS + 1];  // first global tile id of each view
-};
-
-constexpr int BIN_MAXPASS = 6;  // digits of a tile's column and row (at most 30 + 1 bits together)
 
 // Zeroed at the start of each phase: phase 1's counters ...
 struct BinCtl1 {
@@ -145,43 +138,6 @@ struct SrcDepth {
 // --------------------------------------------------------------- records in depth order
 constexpr int REC_IPT = 4;
 constexpr int REC_TILE = OS_THREADS * REC_IPT;
-
-// Tile keys: tile row << xbits | tile column, so that the lowest digits are the
-// column's and a record's counts of them take one addition per column of its
-// mask (or two for a rect of any size, into a difference array).  Grids whose
-// keys fit one digit (at most 8 bits) are sorted by the whole key.
-struct TileKey {
-    int xbits, bits;
-    int npass;
-    int shift[BIN_MAXPASS], width[BIN_MAXPASS];  // digits
-};
-
-static TileKey tile_key(const TileGrid& tg)
-{
-    TileKey k{};
-    int yb = 0;
-    for (int v = 0; v < tg.n; ++v) {
-        while ((1ll << k.xbits) < tg.TX[v]) ++k.xbits;
-        while ((1ll << yb) < tg.TY[v]) ++yb;
-    }
-    k.bits = k.xbits + yb;
-    if (k.bits <= 8) {
-        k.npass = 1;
-        k.width[0] = k.bits > 0 ? k.bits : 1;
-        return k;
-    }
-    // the column's digits, then the row's (a grid of one row or column has none there)
-    for (int part = 0; part < 2; ++part) {
-        const int b = part ? yb : k.xbits, n = (b + 7) / 8, from = part ? k.xbits : 0;
-        for (int i = 0, at = 0; i < n; ++i) {
-            const int w = (b - at + (n - i) - 1) / (n - i);
-            k.shift[k.npass] = from + at;
-            k.width[k.npass++] = w;
-            at += w;
-        }
-    }
-    return k;
-}
 
 // A record in depth order: rect corner x0 | y0 << 16, tile mask (of a whole rect
 // too, up to 8 x 8 tiles; with the top bit of .w set, a larger rect's width and
@@ -328,6 +284,12 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
                     if (e <= dm) atomicAdd(&diff[e], -1);
                 }
             }
+        } else if (tk.linear) {
+            auto add = [&](uint32_t i, int n) { atomicAdd(&diff[i], n); };
+            auto cyc = [&](uint32_t n) { atomicAdd(&s_cycles, n); };
+            const uint32_t a = y0 * (uint32_t)TX + x0;
+            if (masked) count_linear_mask(a, TX, out[k].y, out[k].z, tk.width[0], add, cyc);
+            else count_linear_rect(a, TX, out[k].y, out[k].z, tk.width[0], add, cyc);
         } else if (masked) {
             // pairs of each of the mask's eight columns
             uint32_t any = out[k].y | out[k].z;
@@ -341,13 +303,8 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
             }
         } else {
             // columns x0 .. x0 + w - 1, each h times: cyclic through the digit's values
-            const uint32_t w = out[k].y, h = out[k].z, rem = w & dm, lo = x0 & dm, hi = lo + rem;
-            if (w > dm) atomicAdd(&s_cycles, (w >> tk.width[0]) * h);
-            if (rem) {
-                atomicAdd(&diff[lo], (int)h);
-                if (hi != dm + 1u) atomicAdd(&diff[hi & dm], -(int)h);
-                if (hi > dm + 1u) atomicAdd(&diff[0], (int)h);
-            }
+            count_run(x0, out[k].y, out[k].z, tk.width[0], [&](uint32_t i, int n) { atomicAdd(&diff[i], n); },
+                      [&](uint32_t n) { atomicAdd(&s_cycles, n); });
         }
     }
     __syncthreads();
@@ -389,7 +346,7 @@ struct SrcEmit {
     const unsigned long long* nvis;
     long long P;
     TileGrid tg;
-    int xbits;
+    int linear, xbits;
     BinCtl2* ctl;
     template <int IPT>
     __device__ __forceinline__ uint32_t load(const SegTile& st, int nv, uint32_t* sk, uint32_t* sv,
@@ -402,8 +359,8 @@ struct SrcEmit {
         const uint32_t s_lo = bstart[st.tbase + st.t];
         const uint32_t s_hi = (long long)base + TILE < st.n ? bstart[st.tbase + st.t + 1] : (uint32_t)nvis[st.v] - 1u;
         const int nr = (int)(s_hi - s_lo) + 1;
-        const uint32_t row = 1u << xbits;
-        const uint32_t n_keys = (uint32_t)tg.TY[st.v] << xbits;
+        const uint32_t row = key_row(linear, xbits, tg.TX[st.v]);
+        const uint32_t n_keys = (uint32_t)tg.TY[st.v] * row;
         const uint32_t rbase = (uint32_t)(st.v * P);
         bool bad = false;
         // (whole warps step together: the last round's idle lanes hold an empty mask)
@@ -687,12 +644,13 @@ extern "C" dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64
             ps.hist_next = last ? nullptr : &w.ctl2->hist[0][p + 1][0];
             ps.mask_next = last ? 0u : (1u << tk.width[p + 1]) - 1u;
             if (last) {
+                ps.linear = tk.linear;
                 ps.xbits = tk.xbits;
                 for (int v = 0; v < n_views; ++v) ps.TX[v] = tg.TX[v];
                 ps.ranges = (uint2*)ranges;
                 for (int v = 0; v <= n_views; ++v) ps.toff[v] = tg.off[v];
             }
-            if (p == 0) os_pass<8>(SrcEmit{w.rec, w.poff, w.bstart, w.ctl1->nvis, P, tg, tk.xbits, w.ctl2}, pairs, ps, M_cap, s);
+            if (p == 0) os_pass<8>(SrcEmit{w.rec, w.poff, w.bstart, w.ctl1->nvis, P, tg, tk.linear, tk.xbits, w.ctl2}, pairs, ps, M_cap, s);
             else os_pass<8>(SrcKV{ki, vi}, pairs, ps, M_cap, s);
             ki = ko;
             vi = vo;

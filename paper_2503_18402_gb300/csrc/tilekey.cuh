@@ -1,0 +1,123 @@
+// tilekey.cuh -- sort keys of the pairs: a tile's key within its view, and the
+// counts of a record's lowest key digit.  Host and device code, plain C++.
+#pragma once
+
+#include <stdint.h>
+
+#include "../../include/dashgs.h"
+
+#ifdef __CUDACC__
+#define DG_HD __host__ __device__ __forceinline__
+#else
+#define DG_HD inline
+#endif
+
+namespace dg {
+
+struct TileGrid {
+    int n;
+    int TX[DG_MAX_VIEWS], TY[DG_MAX_VIEWS];
+    int off[DG_MAX_VIEWS + 1];  // first global tile id of each view
+};
+
+constexpr int BIN_MAXPASS = 6;  // digits of a key
+
+// Tile keys: tile row << xbits | tile column, so that the lowest digits are the
+// column's and a record's counts of them take one addition per column of its
+// mask (or two for a rect of any size, into a difference array).  Grids whose
+// keys fit one digit (at most 8 bits) are sorted by the whole key.
+// Linear keys, row * TX + column, serve the grids for which that form fails: with
+// every view one tile wide there is no column digit, and columns and rows whose
+// maxima come from different views may need more than 31 bits together (a view's
+// own grid has at most 2^30 tiles).  A record's lowest digits are then counted
+// run by run.
+struct TileKey {
+    int linear;
+    int xbits, bits;
+    int npass;
+    int shift[BIN_MAXPASS], width[BIN_MAXPASS];  // digits
+};
+
+inline TileKey tile_key(const TileGrid& tg)
+{
+    TileKey k{};
+    int yb = 0, lb = 0;
+    for (int v = 0; v < tg.n; ++v) {
+        while ((1ll << k.xbits) < tg.TX[v]) ++k.xbits;
+        while ((1ll << yb) < tg.TY[v]) ++yb;
+        while ((1ll << lb) < (long long)tg.TX[v] * tg.TY[v]) ++lb;
+    }
+    k.bits = k.xbits + yb;
+    if (k.bits <= 8) {
+        k.npass = 1;
+        k.width[0] = k.bits > 0 ? k.bits : 1;
+        return k;
+    }
+    k.linear = k.xbits == 0 || k.bits > 31;
+    if (k.linear) {
+        k.bits = lb;
+        k.xbits = 0;
+    }
+    // the column's digits, then the row's (a grid of one row has none there), or the linear key's
+    for (int part = 0; part < 2; ++part) {
+        const int b = k.linear ? (part ? 0 : lb) : part ? yb : k.xbits, n = (b + 7) / 8, from = part ? k.xbits : 0;
+        for (int i = 0, at = 0; i < n; ++i) {
+            const int w = (b - at + (n - i) - 1) / (n - i);
+            k.shift[k.npass] = from + at;
+            k.width[k.npass++] = w;
+            at += w;
+        }
+    }
+    return k;
+}
+
+// Key distance of neighbouring tile rows.
+DG_HD uint32_t key_row(int linear, int xbits, int TX) { return linear ? (uint32_t)TX : 1u << xbits; }
+// Tile of a key within its view (row * TX + column).
+DG_HD uint32_t key_tile(uint32_t key, int linear, int xbits, uint32_t TX)
+{
+    return linear ? key : (key >> xbits) * TX + (key & ((1u << xbits) - 1u));
+}
+
+// Counts of the lowest digit of `len` consecutive keys from `a` on, `times` each:
+// cyclic through the digit's values, as a difference array with the full cycles apart.
+template <class Diff, class Cycles>
+DG_HD void count_run(uint32_t a, uint32_t len, uint32_t times, int width, Diff diff, Cycles cycles)
+{
+    const uint32_t dm = (1u << width) - 1u, rem = len & dm, lo = a & dm, hi = lo + rem;
+    if (len > dm) cycles((len >> width) * times);
+    if (rem) {
+        diff(lo, (int)times);
+        if (hi != dm + 1u) diff(hi & dm, -(int)times);
+        if (hi > dm + 1u) diff(0u, (int)times);
+    }
+}
+
+// The same for a record's tiles under linear keys: the mask's bits row by row (lo,
+// hi: eight rows of eight columns), or a rect of w x h tiles.
+template <class Diff, class Cycles>
+DG_HD void count_linear_mask(uint32_t key0, int TX, uint32_t lo, uint32_t hi, int width, Diff diff, Cycles cycles)
+{
+    for (int y = 0; y < 8; ++y) {
+        uint32_t m = ((y < 4 ? lo : hi) >> (8 * (y & 3))) & 255u;
+        uint32_t x = 0;
+        while (m) {
+            while (!(m & 1u)) { m >>= 1; ++x; }
+            uint32_t len = 0;
+            while (m & 1u) { m >>= 1; ++len; }
+            count_run(key0 + (uint32_t)(y * TX) + x, len, 1u, width, diff, cycles);
+            x += len;
+        }
+    }
+}
+template <class Diff, class Cycles>
+DG_HD void count_linear_rect(uint32_t key0, int TX, uint32_t w, uint32_t h, int width, Diff diff, Cycles cycles)
+{
+    if (w == (uint32_t)TX) {  // whole rows follow one another
+        count_run(key0, w * h, 1u, width, diff, cycles);
+        return;
+    }
+    for (uint32_t y = 0; y < h; ++y) count_run(key0 + y * (uint32_t)TX, w, 1u, width, diff, cycles);
+}
+
+}  // namespace dg
