@@ -194,12 +194,12 @@ DG_API dg_status dg_bin_count(const float* depth, const int32_t* tiles, int64_t 
  * of dg_project) gets pairs only for the mask's tiles.
  * Out: gid    [M_cap] uint32, record index v * P + i of each sorted pair;
  *      ranges [2 * total tiles] uint32, [start, end) of each tile's list;
- *      status (device int32): 0, or DG_ERR_CAPACITY when M > M_cap, in which
- *              case gid is untouched and every range is empty, or
- *              DG_ERR_TIMEOUT when a bounded wait between thread blocks
- *              gave up (lists not valid; does not happen when the device
- *              runs the launch to completion), or DG_ERR_CUDA when the records'
- *              pairs are not those counted in phase 1 (every range is empty).
+ *      status (device int32): 0, or an error, with which every range is empty:
+ *              DG_ERR_CAPACITY when M > M_cap (gid is untouched),
+ *              DG_ERR_TIMEOUT when a bounded wait between thread blocks gave up
+ *              (does not happen when the device runs the launch to completion),
+ *              DG_ERR_CUDA when the records' pairs are not those counted in
+ *              phase 1 or lie outside the grid (gid holds nothing to be read).
  * feat/radius are dg_project's outputs for the same P and cameras. */
 DG_API dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64_t P, const dg_camera* cams,
                       int32_t n_views, int32_t tile, void* ws, size_t ws_bytes, int64_t M_cap, uint32_t* gid,

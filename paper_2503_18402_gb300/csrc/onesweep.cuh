@@ -411,8 +411,13 @@ k_os_pass(Src src, Segs sg, OsPass ps)
             st_relaxed(look + d0, LbWord<Word>::inc((Word)before + (Word)total));
         }
         const uint32_t at = (uint32_t)(ex >> 32) + before;
-        // (always inside the view's items, unless a wait gave up in this pass or before)
-        if ((unsigned long long)at + total > (unsigned long long)st.n) s_bad = 1;
+        // (always inside the view's items, unless a wait gave up in this pass or before
+        // or the digit counts are not those of the items; the tile is dropped then, so
+        // what the pass leaves is not to be used)
+        if ((unsigned long long)at + total > (unsigned long long)st.n) {
+            s_bad = 1;
+            atomicCAS(ps.err, 0, DG_ERR_CUDA);
+        }
         gstart[d0] = (uint32_t)st.off + at - (uint32_t)ex;
     }
     __syncthreads();

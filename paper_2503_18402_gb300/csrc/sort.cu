@@ -431,16 +431,20 @@ struct SrcEmit {
     }
 };
 
-// Ranges from their (complement of the start, end) form, and the call's status.
+// Ranges from their (complement of the start, end) form, and the call's status.  With
+// any error every range is empty: gid may hold words of an earlier call then, and the
+// passes that read the lists are launched before the host sees the status.
 __global__ void k_ranges_final(uint2* __restrict__ ranges, int n_tiles, const long long* M, long long M_cap,
                                const int* err1, const BinCtl2* ctl, int* status)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int st = *M > M_cap ? DG_ERR_CAPACITY : (*err1 != 0 ? *err1 : ctl->err);
     if (i < n_tiles) {
         const uint2 r = ranges[i];
-        if (r.y != 0u) ranges[i].x = ~r.x;
+        if (st != 0) ranges[i] = make_uint2(0u, 0u);
+        else if (r.y != 0u) ranges[i].x = ~r.x;
     }
-    if (i == 0) *status = *M > M_cap ? DG_ERR_CAPACITY : (*err1 != 0 ? *err1 : ctl->err);
+    if (i == 0) *status = st;
 }
 
 // Workspace layout (offsets 256-byte aligned).  The pair count and the
