@@ -89,11 +89,14 @@ class Rasterizer:
         # mixed-precision copy of the records read by the render passes (opts.record == 1)
         self.packed = (torch.empty(n * capi.PACKED_RECORD_BYTES, dtype=torch.uint8, device=d)
                        if self.opts.record == 1 else None)
-        self.M_dev = torch.zeros(1, dtype=torch.int64, device=d)
-        # pinned landing slot of the pair count: one async copy and one event wait
-        self.M_host = torch.zeros(1, dtype=torch.int64).pin_memory()
-        self.M_event = torch.cuda.Event()
-        self.status = torch.zeros(1, dtype=torch.int32, device=d)
+        if not hasattr(self, "count_status"):  # (kept when the records grow: the last frame's status is still to be read)
+            # pair count (int64) and status (int32 in the second word) side by side
+            self.count_status = torch.zeros(2, dtype=torch.int64, device=d)
+            self.M_dev = self.count_status[0:1]
+            self.status = self.count_status[1:2].view(torch.int32)[0:1]
+            # pinned landing slot of both: one async copy and one event wait
+            self.M_host = torch.zeros(2, dtype=torch.int64).pin_memory()
+            self.M_event = torch.cuda.Event()
         self.N_cap = N
         self.ws = None
 
@@ -164,11 +167,27 @@ class Rasterizer:
         return Frame(P=P, cams=cams, img=f["img"], T=f["T"], last=f["last"], M=-1, flat_img=f["img"],
                      flat_T=f["T"], flat_last=f["last"])
 
+    # ------------------------------------------------------------ errors
+    @staticmethod
+    def _raise_for(word):
+        """Raises for a status word of the binning (its low 32 bits); a capacity
+        overflow is the callers' to handle."""
+        st = (word & 0xffffffff) - ((word & 0x80000000) << 1)
+        if st not in (capi.DG_OK, capi.DG_ERR_CAPACITY):
+            raise capi.DashGSError(st, "the binning of an earlier frame failed: its lists were left empty")
+
+    def check(self):
+        """Waits for the last frame and raises if its binning failed."""
+        if self.N_cap >= 0:
+            torch.cuda.synchronize(self.device)
+            self._raise_for(int(self.status.item()))
+
     # ------------------------------------------------------------ passes
     def forward(self, params: torch.Tensor, P: int, cams, stream=None, examined: bool = False) -> Frame:
         """Project, bin, sort and composite P Gaussians of the planar
         [59, stride] float32 tensor ``params`` into one camera or a list of
-        cameras (at most 16)."""
+        cameras (at most 16).  A frame whose binning failed raises in the next
+        call or in check()."""
         assert params.dtype == torch.float32 and params.shape[0] == NPARAM and params.stride(1) == 1
         cams = [cams] if isinstance(cams, capi.Camera) else list(cams)
         V = len(cams)
@@ -188,7 +207,7 @@ class Rasterizer:
         capi.dg_bin_count(self.depth, self.tiles, P, V, self.ws, self.ws.numel(), self.M_cap, self.M_dev, stream)
         self._mark("bin_count")
         with torch.cuda.stream(stream):
-            self.M_host.copy_(self.M_dev, non_blocking=True)
+            self.M_host.copy_(self.count_status, non_blocking=True)
         self.M_event.record(stream)
         # the pair sort is queued before the count reaches the host, so the GPU
         # runs on while the host waits; when the pairs exceed the capacity it
@@ -197,7 +216,11 @@ class Rasterizer:
                          self.ranges, self.status, stream)
         self._mark("bin_sort")
         self.M_event.synchronize()
-        M = int(self.M_host[0])
+        # the status word is the previous call's (this call's pair sort is still
+        # running): a failed binning, whose frame shows the background only, is
+        # reported one call later, without a second wait for every frame
+        M, st = self.M_host.tolist()
+        self._raise_for(st)
         if M > self.M_cap:
             self._ensure_ws(P, V, int(M * self.headroom) + 1024)
             capi.dg_bin_count(self.depth, self.tiles, P, V, self.ws, self.ws.numel(), self.M_cap, self.M_dev, stream)

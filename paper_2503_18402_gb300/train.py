@@ -309,6 +309,8 @@ class Trainer:
             status, M = g_prev.result(slot)
             sz = g_prev.sizes[0]
             self.M_hint[sz] = max(self.M_hint.get(sz, 0), M)
+            if status not in (capi.DG_OK, capi.DG_ERR_CAPACITY):
+                raise capi.DashGSError(status, "the binning of a replayed step failed")
             if status != 0:  # pair capacity exceeded: that step made no update
                 self.skipped_steps += 1
                 self.graphs.pop(g_prev.key, None)
@@ -451,6 +453,8 @@ class Trainer:
                                       s=round(time.perf_counter() - t0, 2))), flush=True)
         torch.cuda.synchronize()
         self._check_pending(keep=0)
+        for rz in self.tuner.rz.values():
+            rz.check()
         return dict(seconds=time.perf_counter() - t0, schedule_init_s=self.init_schedule_s, P_final=self.P,
                     iters_per_factor={str(k): v for k, v in sorted(res_hist.items())},
                     render_shapes=self.tuner.summary(), views_per_step=self.V, steps=self.n_steps,

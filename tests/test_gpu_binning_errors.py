@@ -41,3 +41,32 @@ def test_a_mask_outside_the_grid_leaves_no_lists(W, H):
     capi.dg_bin_sort(rz.feat, rz.radius, P, cam, 1, B, rz.ws, rz.ws.numel(), rz.M_cap, rz.gid, rz.ranges, rz.status)
     r = rz.ranges.cpu().numpy().view(np.uint32).astype(np.int64)
     assert int(rz.status.item()) == 0 and int((r[:, 1] - r[:, 0]).sum()) == fr.M
+
+
+def test_the_rasterizer_raises_for_a_failed_binning():
+    """A status word that a failed binning left is raised by the next frame and by
+    check(); a capacity overflow is not, and a frame that binned clears it."""
+    P, W, H = 500, 64, 48
+    cam = make_camera(np.asarray(synth.look_at(np.array([0.0, -4.0, 0.0])), np.float32).reshape(-1),
+                      synth.intrinsics(W, H, 45.0), W, H)
+    prm = torch.from_numpy(np.ascontiguousarray(synth.random_gaussians(P, 5).T.astype(np.float32))).cuda()
+    rz = Rasterizer("cuda", capi.raster_opts(tile=8))
+    rz.check()
+    want = rz.forward(prm, P, cam).img.clone()
+    rz.check()
+    for code in (capi.DG_ERR_TIMEOUT, capi.DG_ERR_CUDA):
+        rz.status.fill_(code)
+        with pytest.raises(capi.DashGSError) as e:
+            rz.check()
+        assert e.value.status == code
+        with pytest.raises(capi.DashGSError) as e:
+            rz.forward(prm, P, cam)
+        assert e.value.status == code
+        assert torch.equal(rz.forward(prm, P, cam).img, want)  # the frame before this one binned
+    rz.status.fill_(capi.DG_ERR_CAPACITY)
+    rz.check()
+    assert torch.equal(rz.forward(prm, P, cam).img, want)
+    rz.status.fill_(capi.DG_ERR_CUDA)
+    big = torch.cat([prm, prm], 1)
+    with pytest.raises(capi.DashGSError):  # also when the record buffers grow
+        rz.forward(big, 2 * P, cam)
