@@ -94,7 +94,7 @@ struct DensCtl {
     uint32_t hist[3][SEL_BINS];
     uint32_t ctr;
     int32_t err;
-    long long n_keep;
+    long long n_keep, n_all;  // survivors; with the appended Gaussians
 };
 
 // Sort key of a score (>= 0): ascending key = descending score.
@@ -187,7 +187,7 @@ constexpr int PL_TILE = SEL_THREADS * PL_IPT;
 __global__ void __launch_bounds__(SEL_THREADS)
 k_places(uint8_t* __restrict__ flags, const float* __restrict__ score, int P, int mode, unsigned long long n_sel,
          DensCtl* ctl, uint64_t* __restrict__ look, int n_tiles, uint32_t* __restrict__ keep_pos,
-         uint32_t* __restrict__ app_pos, uint32_t* __restrict__ sel_rank, long long* __restrict__ P_out)
+         uint32_t* __restrict__ app_pos, uint32_t* __restrict__ sel_rank)
 {
     __shared__ uint32_t s_bin, s_sum[SEL_THREADS / 32];
     __shared__ unsigned long long s_below;
@@ -233,7 +233,7 @@ k_places(uint8_t* __restrict__ flags, const float* __restrict__ score, int P, in
             uint64_t e = 0;
             if (lane == 0) st_relaxed(look + t, (t == 0 ? kLbInc : kLbAgg) | tot);
             if (t > 0) {
-                if (!os_lookback_warp(look, t, &e, lane) && lane == 0) ctl->err = DG_ERR_TIMEOUT;
+                if (!os_lookback_warp(look, t, &e, lane) && lane == 0) atomicExch(&ctl->err, DG_ERR_TIMEOUT);
                 if (lane == 0) st_relaxed(look + t, kLbInc | (e + tot));
             }
             if (lane == 0) s_ex[0] = e;
@@ -275,7 +275,7 @@ k_places(uint8_t* __restrict__ flags, const float* __restrict__ score, int P, in
         uint64_t e = 0;
         if (lane == 0) st_relaxed(lk + t, (t == 0 ? kLbInc : kLbAgg) | mine);
         if (t > 0) {
-            if (!os_lookback_warp(lk, t, &e, lane) && lane == 0) ctl->err = DG_ERR_TIMEOUT;
+            if (!os_lookback_warp(lk, t, &e, lane) && lane == 0) atomicExch(&ctl->err, DG_ERR_TIMEOUT);
             if (lane == 0) st_relaxed(lk + t, kLbInc | (e + mine));
         }
         if (lane == 0) s_ex[1 + warp] = e;
@@ -300,7 +300,7 @@ k_places(uint8_t* __restrict__ flags, const float* __restrict__ score, int P, in
         const uint64_t all = s_ex[2] + tot[1];
         const long long nk = (long long)(s_ex[1] + tot[0]);
         ctl->n_keep = nk;
-        *P_out = ctl->err != 0 ? (long long)ctl->err : nk + (long long)(all & k31) + (long long)(all >> 31);
+        ctl->n_all = nk + (long long)(all & k31) + (long long)(all >> 31);
     }
 }
 
@@ -323,9 +323,11 @@ k_densify_write(const float* __restrict__ prm, const float* __restrict__ m, cons
                 long long stride, int P, const uint8_t* __restrict__ flags, const uint32_t* __restrict__ keep_pos,
                 const uint32_t* __restrict__ app_pos, const uint32_t* __restrict__ sel_rank, const DensCtl* ctl,
                 const float* __restrict__ noise, float log_div, float* __restrict__ dp, float* __restrict__ dm,
-                float* __restrict__ dv, long long dstride)
+                float* __restrict__ dv, long long dstride, long long* __restrict__ P_out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    // (here, not in the kernel of the places: only behind it is its error word final)
+    if (i == 0 && blockIdx.y == 0) *P_out = ctl->err != 0 ? (long long)ctl->err : ctl->n_all;
     if (i >= P || ctl->err != 0) return;  // (a wait gave up: the places are not known)
     const uint8_t f = flags[i];
     const bool sel = f & F_SEL, split = sel && (f & F_SPLIT), keep = (f & F_KEEP) && !split;
@@ -517,11 +519,11 @@ extern "C" dg_status dg_densify_apply(const float* params, const float* m, const
     }
     const int nt = (int)((P + dg::PL_TILE - 1) / dg::PL_TILE);
     dg::k_places<<<nt, dg::SEL_THREADS, 0, s>>>(w.flags, w.score, (int)P, mode, (unsigned long long)n_sel, w.ctl, w.look,
-                                              nt, w.keep_pos, w.app_pos, w.sel_rank, (long long*)P_out);
+                                              nt, w.keep_pos, w.app_pos, w.sel_rank);
     const dim3 grid((unsigned)((P + 255) / 256), (DG_NPARAM + dg::DW_ROWS - 1) / dg::DW_ROWS);
     dg::k_densify_write<<<grid, 256, 0, s>>>(params, m, v, (long long)stride, (int)P, w.flags, w.keep_pos, w.app_pos,
                                              w.sel_rank, w.ctl, noise, (float)log(1.6), dst_params, dst_m, dst_v,
-                                             (long long)dst_stride);
+                                             (long long)dst_stride, (long long*)P_out);
     dg_note_launch(2);
     return dg_check_launch("densify_apply");
 }
