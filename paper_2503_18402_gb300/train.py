@@ -420,7 +420,10 @@ class Trainer:
         noise = torch.randn((max(n_sel, 1), 2, 3), generator=self.gen, device=self.dev)
         capi.dg_densify_apply(b["p"], b["m"], b["v"], self.cap, P, n_cand, budget, noise, self.dws, self.dws.numel(),
                               dst["p"], dst["m"], dst["v"], self.cap, self.P_out, self.stream)
-        self.P = int(self.P_out.item())
+        P_new = int(self.P_out.item())
+        if P_new < 0:  # an error word instead of a count: nothing was written
+            raise capi.DashGSError(P_new, "the densification failed")
+        self.P = P_new
         self.cur = 1 - self.cur
         self.acc.zero_(); self.den.zero_(); self.maxr.zero_()
         self.history.append(dict(iter=k, P=self.P, n_keep=n_keep, n_cand=n_cand, budget=budget))
