@@ -172,7 +172,8 @@ struct RViews {
 // Head of the render workspace.  The forward writes the split plan here and
 // in the arrays after it; the backward of the same batch reads it.
 struct RHdr {
-    int cnt_prod, cnt_fwd, cnt_bwd, cnt_pad;  // work counters of the three persistent launches
+    int cnt_prod, cnt_fwd, cnt_bwd;           // work counters of the three persistent launches
+    int colours;                              // set by k_render_fwd_w: 1 it ran, 2 it met a colour that is not finite
     int planned;                              // 1: items/sitems hold a split plan
     int L;                                    // chunk length of that plan
     int n_items, n_slots;                     // items (all chunks), chunks of split tiles
@@ -959,6 +960,12 @@ __device__ inline Item next_item_warp(int* counter, int count, const int4* list,
     return it;
 }
 
+// True unless a colour channel is infinite or NaN.
+__device__ __forceinline__ bool finite_colour(float r, float g, float b)
+{
+    return fmaf(b, 0.f, fmaf(g, 0.f, r * 0.f)) == 0.f;
+}
+
 // Reciprocal on the special-function unit (rcp.approx: about 1 ulp; exactly 1 for 1).
 __device__ __forceinline__ float rcp_approx(float x)
 {
@@ -1004,31 +1011,35 @@ __device__ __forceinline__ float rcp_approx(float x)
 // block -> 3.20 ms with the row's dL/dC in registers instead of read from shared
 // memory per group (12 blocks of 64 threads per SM; 9, 10, 11 blocks 3.21, 3.23,
 // 3.20 ms).
-template <int REC>
-__global__ void __launch_bounds__(64, 12)
-k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
-                const uint2* __restrict__ ranges, RViews rv, RHdr* hdr, const int4* __restrict__ items, Slots sl,
-                const uint8_t* __restrict__ flags, long long flags_cap,
-                const float* __restrict__ Tfin, const int* __restrict__ lastin,
-                const float* __restrict__ dLdimg, float4* __restrict__ grad2d)
-{
-    constexpr int B = 8, NPIX = 64;
+struct EpShared {
     // staged entry pairs: (u, u', v, v'), (a, a', b, b') the forward's prescaled
     // conic, (c, c', log2 o, log2 o'), (r, r', g, g'), (b, b', list positions)
-    __shared__ float4 s_pair[2][kEpRing / 2 * kPairW];
-    __shared__ float4 s_k[2][kEpRing];           // A, B, C, 1/o
-    __shared__ uint32_t s_g[2][kEpRing];
-    __shared__ float4 s_m[2][kEpG / 2 * kEpPitch];  // [pair][pixel] (dp, dp', wT, wT')
-    __shared__ float4 s_px[2][32];               // per pixel dL/dC
+    float4 pair[2][kEpRing / 2 * kPairW];
+    float4 k[2][kEpRing];                // A, B, C, 1/o
+    uint32_t g[2][kEpRing];
+    float4 m[2][kEpG / 2 * kEpPitch];    // [pair][pixel] (dp, dp', wT, wT')
+    float4 px[2][32];                    // per pixel dL/dC
+};
+
+// APART: some staged colour may be infinite or NaN.
+template <int REC, bool APART>
+__device__ __forceinline__ void
+render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
+              const uint2* __restrict__ ranges, RViews rv, RHdr* hdr, const int4* __restrict__ items, Slots sl,
+              const uint8_t* __restrict__ flags, long long flags_cap,
+              const float* __restrict__ Tfin, const int* __restrict__ lastin,
+              const float* __restrict__ dLdimg, float4* __restrict__ grad2d, EpShared& sh)
+{
+    constexpr int B = 8, NPIX = 64;
     const float bg0 = rv.bg0, bg1 = rv.bg1, bg2 = rv.bg2;
     const bool planned = hdr->planned != 0 && items != nullptr;
     const int L = planned ? hdr->L : INT_MAX;
     const int count = planned ? hdr->n_items : rv.total;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    float4* const sp = s_pair[wp];
-    float4* const sm = s_m[wp];
-    float4* const wk = s_k[wp];
-    uint32_t* const wg = s_g[wp];
+    float4* const sp = sh.pair[wp];
+    float4* const sm = sh.m[wp];
+    float4* const wk = sh.k[wp];
+    uint32_t* const wg = sh.g[wp];
     const uint32_t above = ~((2u << lane) - 1u);  // lanes behind this one in the list
     for (;;) {
     int blk = 0;
@@ -1067,13 +1078,13 @@ k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
         }
     }
     __syncwarp();
-    s_px[wp][lane] = make_float4(g0, g1, g2, 0.f);
+    sh.px[wp][lane] = make_float4(g0, g1, g2, 0.f);
     __syncwarp();
     // phase B: dL/dC of the 8 pixels of this lane's row
     float gpr[8], gpg[8], gpb[8];
 #pragma unroll
     for (int px = 0; px < 8; ++px) {
-        const float4 c = s_px[wp][8 * (lane >> 3) + px];
+        const float4 c = sh.px[wp][8 * (lane >> 3) + px];
         gpr[px] = c.x; gpg[px] = c.y; gpb[px] = c.z;
     }
     const int top = min(__reduce_max_sync(0xffffffffu, lastp), hi);
@@ -1169,6 +1180,10 @@ k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
                 f2_unpack(gu, gc0, gc1);
                 const bool b0 = __float_as_int(bp.z) < lastp && p0 <= 0.f && e0 >= kLog2AlphaMin;
                 const bool b1 = __float_as_int(bp.w) < lastp && p1 <= 0.f && e1 >= kLog2AlphaMin;
+                if (APART) {  // the colour of an entry that is not blended stays out of g . S
+                    if (!b0) gc0 = 0.f;
+                    if (!b1) gc1 = 0.f;
+                }
                 const float r0 = ex2_approx(e0), r1 = ex2_approx(e1);
                 const float a0 = b0 ? fminf(kAlphaMax, r0) : 0.f, a1 = b1 ? fminf(kAlphaMax, r1) : 0.f;
                 const float i0 = rcp_approx(1.f - a0), i1 = rcp_approx(1.f - a1);
@@ -1266,6 +1281,25 @@ k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
     }  // work items
 }
 
+// The walk for finite colours unless the forward met others, or was another pass
+// (then nothing is known): a weight of 0 leaves g . S alone only where the colour is
+// finite, and keeping the others out takes two more instructions per step.  On 16
+// views of 1237x822, 480k Gaussians, mixed records: 3.12 ms without the test, 3.20
+// with it in every step, 3.16 with two walks side by side in one body, 3.05 with a
+// body for each form.
+template <int REC>
+__global__ void __launch_bounds__(64, 12)
+k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
+                const uint2* __restrict__ ranges, RViews rv, RHdr* hdr, const int4* __restrict__ items, Slots sl,
+                const uint8_t* __restrict__ flags, long long flags_cap,
+                const float* __restrict__ Tfin, const int* __restrict__ lastin,
+                const float* __restrict__ dLdimg, float4* __restrict__ grad2d)
+{
+    __shared__ EpShared sh;
+    if (hdr->colours == 1) render_bwd_ep<REC, false>(feat, gid, ranges, rv, hdr, items, sl, flags, flags_cap, Tfin, lastin, dLdimg, grad2d, sh);
+    else render_bwd_ep<REC, true>(feat, gid, ranges, rv, hdr, items, sl, flags, flags_cap, Tfin, lastin, dLdimg, grad2d, sh);
+}
+
 // Forward of 8x8 tiles with one pixel per thread, each warp on its own: a work
 // item is one 8x4 block of a tile (or of a chunk of a split tile), taken per
 // warp from the counter (the same compositing as k_render_fwd, pixel for
@@ -1288,6 +1322,41 @@ k_render_bwd_ep(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
 // a branch per entry -> 2.27 ms -> 2.09 ms with one address per staged pair and
 // only the facing edges in the cull (on four of the views 781M -> 595M -> 543M
 // warp instructions).
+//
+// An entry whose colour is not finite leaves no finite sum in any lane, whatever its
+// weight; such a block's colours are formed again, entry by entry and only from those
+// the pixel blends (a test of every batch's colours cost 0.6%, a second round of the
+// walk's own loop 2.3%, this call 0.5% of the pass when all colours are finite).
+template <int REC>
+__device__ __noinline__ float3 blended_colour(const void* feat, const uint32_t* gid, int count, float pxc, float pyc,
+                                              float T, bool on)
+{
+    float3 c = make_float3(0.f, 0.f, 0.f);
+    for (int j = 0; j < count && __any_sync(0xffffffffu, on); ++j) {
+        float4 ga, gb;
+        float gc;
+        load_record<REC>(feat, gid[j], ga, gb, gc);
+        // (the roundings of the walk)
+        const float dx = __fadd_rn(ga.x, -pxc), dy = __fadd_rn(ga.y, -pyc);
+        const float p = fmaf(dx, fmaf(-kLog2e * ga.w, dy, __fmul_rn(-0.5f * kLog2e * ga.z, dx)),
+                             __fmul_rn(__fmul_rn(-0.5f * kLog2e * gb.x, dy), dy));
+        const float e = __fadd_rn(p, __log2f(gb.y));
+        if (!on || !(gb.y >= kAlphaMin) || !(p <= 0.f && e >= kLog2AlphaMin)) continue;
+        const float a = fminf(kAlphaMax, ex2_approx(e));
+        const float Tn = fmaf(-a, T, T);
+        if (Tn < kTMin) {
+            on = false;
+            continue;
+        }
+        const float w = __fmul_rn(a, T);
+        c.x = fmaf(w, gb.z, c.x);
+        c.y = fmaf(w, gb.w, c.y);
+        c.z = fmaf(w, gc, c.z);
+        T = Tn;
+    }
+    return c;
+}
+
 template <bool PROD, int REC>
 // (16 blocks of 64 threads per SM, 64 registers: 0.366 -> 0.353 ms against the
 // compiler's 56-register choice of 18 blocks)
@@ -1313,6 +1382,7 @@ k_render_fwd_w(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
     auto pos_of = [&](int slot) { return __float_as_int(sp[(slot >> 1) * kPairW + 3 + (slot & 1)].w); };
     const uint32_t lt = (1u << lane) - 1u;
     const float kNever = __int_as_float(0x7f800000);  // threshold of a pixel that takes no entry
+    if (!PROD && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&hdr->colours, 1);
     for (;;) {
     int blk = 0;
     const Item it = next_item_warp(counter, count, list, rv, &blk);
@@ -1447,6 +1517,14 @@ k_render_fwd_w(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
         __syncwarp();
     }
     if (Tend >= 0.f) T = Tend;
+    if (!PROD && __any_sync(0xffffffffu, !finite_colour(c0, c1, c2))) {
+        if (lane == 0) atomicOr(&hdr->colours, 2);
+        float T0 = 1.f;
+        for (int c = 0; split && c < it.c; ++c) T0 *= sl.prod[(size_t)(it.slot0 + c) * NPIX + p];
+        const float3 c = blended_colour<REC>(feat, gid + rg.x + lo, hi - lo, pxc, pyc, T0,
+                                             x < W && y < H && !(T0 < kTMin));
+        c0 = c.x; c1 = c.y; c2 = c.z;
+    }
     if (split) {
         const size_t s0 = (size_t)(it.slot0 + it.c) * NPIX + (size_t)p;
         if (PROD) {

@@ -1,0 +1,59 @@
+"""Colours that are not finite reach only the pixels that blend them, and through
+those only the gradients of the entries these pixels blend, against the FP64
+oracle fed the same records: where the oracle is finite the kernels are finite
+and close, and where it is not they are not."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+from paper_2503_18402_gb300 import capi, synth  # noqa: E402
+from paper_2503_18402_gb300.raster import Rasterizer  # noqa: E402
+from tests import _gpu as G  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _same(got, want, tol):
+    """Finite in the same places, and there within tol(want)."""
+    fin = np.isfinite(want)
+    np.testing.assert_array_equal(np.isfinite(got), fin)
+    assert (np.abs(got[fin] - want[fin]) <= tol(np.abs(want[fin]))).all()
+    return fin
+
+
+@pytest.mark.parametrize("tile,ppt", [(8, 1), (8, 2), (16, None)])
+@pytest.mark.parametrize("split", [-1, 5, 32])
+@pytest.mark.parametrize("n", [3, 40, 161])
+def test_nonfinite_colours_stay_with_their_pixels(n, split, tile, ppt):
+    W, H, bg = 29, 21, (0.2, 0.4, 0.1)
+    g = synth.random_gaussians(n, 700 + n)
+    rng = np.random.default_rng(n)
+    g[:, 0:2] *= 0.6
+    g[:, 3:6] = rng.normal(-2.0, 0.4, size=(n, 3))
+    for i, (ch, val) in enumerate([(0, np.nan), (1, np.inf), (2, -np.inf)]):  # channels of three Gaussians
+        g[(i * n) // 3, 11 + ch] = val
+    cam = synth.camera_cfg0(W, H, 4.0)
+    k = oracle.consts()
+    rz = Rasterizer("cuda", capi.raster_opts(tile=tile, bg=bg, split_len=split), ppt_fwd=ppt, ppt_bwd=ppt)
+    params = G.gpu_params(g)
+    fr = rz.forward(params, n, G.gpu_camera(cam), examined=True)
+    feat = G.np_(rz.feat[:n]).astype(np.float64)[:, :9]
+    assert (~np.isfinite(feat[:, 6:9])).any(1).sum() >= 2
+    gid = G.np_(rz.gid[: fr.M]).view(np.uint32)
+    n_tiles = -(-W // tile) * -(-H // tile)
+    ranges = G.np_(rz.ranges[:n_tiles]).view(np.uint32).reshape(-1)
+    orf = oracle.render_fwd(feat, W, H, tile, gid, ranges, G.f32(bg), k)
+    fin = _same(G.np_(fr.img), orf["img"], lambda a: 1e-5)
+    if n > 3:
+        assert fin.any() and not fin.all()
+    np.testing.assert_array_equal(G.np_(fr.last), orf["last"])
+    np.testing.assert_array_equal(G.np_(rz.examined), orf["examined"])
+    np.testing.assert_array_equal(G.np_(rz.blended), orf["blended"])
+    dL = (rng.normal(size=(3, H, W)) / (3 * H * W)).astype(np.float32)
+    rz.backward_render(fr, torch.from_numpy(dL).cuda())
+    og2 = oracle.render_bwd(feat, W, H, tile, gid, ranges, G.f32(bg), k, dL.astype(np.float64))
+    fin = _same(G.np_(rz.grad2d[:n])[:, :9], og2, lambda a: 1e-4 * a + 1e-6)
+    if n > 3:
+        assert fin[:, :6].all(1).any() and not fin.all()
