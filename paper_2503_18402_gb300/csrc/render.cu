@@ -1381,7 +1381,10 @@ k_render_fwd_w(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
     float4* const sp = s_pair[wp];
     auto pos_of = [&](int slot) { return __float_as_int(sp[(slot >> 1) * kPairW + 3 + (slot & 1)].w); };
     const uint32_t lt = (1u << lane) - 1u;
-    const float kNever = __int_as_float(0x7f800000);  // threshold of a pixel that takes no entry
+    // threshold of a pixel that takes no entry: NaN, which no alpha reaches, not even an
+    // infinite opacity's
+    const float kNever = __int_as_float(0x7fc00000);
+    auto never = [](float t) { return t != t; };
     if (!PROD && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&hdr->colours, 1);
     for (;;) {
     int blk = 0;
@@ -1415,7 +1418,7 @@ k_render_fwd_w(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
             T = 1.f;
         }
     }
-    bool alldone = __all_sync(0xffffffffu, thr == kNever);
+    bool alldone = __all_sync(0xffffffffu, never(thr));
     const f32x2 npx = f2_pack(-pxc, -pxc), npy = f2_pack(-pyc, -pyc);
     // the Gaussian indices of a batch are loaded one batch ahead, so a batch
     // waits only for its records
@@ -1446,7 +1449,7 @@ k_render_fwd_w(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
         if ((cnt & 1) && lane == 0) {  // the last pair's second half: an entry no pixel blends
             float4* q = sp + (cnt >> 1) * kPairW;
             float* f = (float*)q + 1;
-            f[0] = 0.f; f[2] = 0.f; f[4] = 0.f; f[6] = 0.f; f[8] = 0.f; f[10] = -kNever;
+            f[0] = 0.f; f[2] = 0.f; f[4] = 0.f; f[6] = 0.f; f[8] = 0.f; f[10] = __int_as_float(0xff800000);
             q[4] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         __syncwarp();
@@ -1488,7 +1491,7 @@ k_render_fwd_w(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
                     T1 = T0;
                     thr = kNever;
                 }
-                leave = __all_sync(0xffffffffu, thr == kNever);
+                leave = __all_sync(0xffffffffu, never(thr));
             }
             if (!PROD) {
                 const float4 q0 = q[3], q1 = q[4];
@@ -1513,7 +1516,7 @@ k_render_fwd_w(const void* __restrict__ feat, const uint32_t* __restrict__ gid,
                 }
             }
         }
-        alldone = __all_sync(0xffffffffu, thr == kNever);
+        alldone = __all_sync(0xffffffffu, never(thr));
         __syncwarp();
     }
     if (Tend >= 0.f) T = Tend;

@@ -57,3 +57,34 @@ def test_nonfinite_colours_stay_with_their_pixels(n, split, tile, ppt):
     fin = _same(G.np_(rz.grad2d[:n])[:, :9], og2, lambda a: 1e-4 * a + 1e-6)
     if n > 3:
         assert fin[:, :6].all(1).any() and not fin.all()
+
+
+@pytest.mark.parametrize("split", [-1, 2])
+def test_infinite_opacity_does_not_restart_a_stopped_pixel(split):
+    """Records of infinite opacity blend at the clamp.  Behind a wide, a small and a
+    second wide entry the pixels under the small one stop at the first of them, the
+    others a step later; the stopped ones examine nothing more."""
+    W, H, n = 13, 11, 6
+    g = synth.random_gaussians(n, 41)
+    g[:, 0:2] *= 0.1
+    g[:, 3:6] = 0.5
+    cam = synth.camera_cfg0(W, H, 4.0)
+    gcam = G.gpu_camera(cam)
+    k = oracle.consts()
+    rz = Rasterizer("cuda", capi.raster_opts(tile=8, split_len=split, tight_bins=0), ppt_fwd=1, ppt_bwd=1)
+    fr = rz.forward(G.gpu_params(g), n, gcam)
+    order = [int(i) for i in rz.gid[:n]]  # of the first tile, and of all: every record is wide
+    for i, o in zip(order, (0.9, 0.98, 0.3) + (float("inf"),) * 3):
+        rz.feat[i, :6] = torch.tensor([6.1, 5.2, 1e-4, 0.0, 1e-4, o])
+    rz.feat[order[1], :5] = torch.tensor([3.2, 2.7, 1.0, 0.0, 1.0])
+    img, T = torch.empty_like(fr.img), torch.empty_like(fr.T)
+    last, ex, bl = (torch.empty_like(fr.last) for _ in range(3))
+    capi.dg_render_fwd(rz.feat, rz.gid, rz.ranges, gcam, 1, rz.opts_fwd, img, T, last, ex, bl, rz.rws, rz.rws.numel())
+    feat = G.np_(rz.feat[:n]).astype(np.float64)[:, :9]
+    orf = oracle.render_fwd(feat, W, H, 8, G.np_(rz.gid[: fr.M]).view(np.uint32),
+                            G.np_(rz.ranges[:4]).view(np.uint32).reshape(-1), np.zeros(3), k)
+    assert set(np.unique(orf["examined"])) == {4, 5}
+    np.testing.assert_array_equal(G.np_(last), orf["last"])
+    np.testing.assert_array_equal(G.np_(ex), orf["examined"])
+    np.testing.assert_array_equal(G.np_(bl), orf["blended"])
+    assert np.abs(G.np_(img) - orf["img"]).max() <= 1e-5
