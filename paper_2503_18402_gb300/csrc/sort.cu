@@ -139,10 +139,7 @@ struct SrcDepth {
 constexpr int REC_IPT = 4;
 constexpr int REC_TILE = OS_THREADS * REC_IPT;
 
-// A record in depth order: rect corner x0 | y0 << 16, tile mask (of a whole rect
-// too, up to 8 x 8 tiles; with the top bit of .w set, a larger rect's width and
-// height), and its index in the view.
-constexpr uint32_t kRectFlag = 0x80000000u;
+// A record in depth order: its tiles (RecTiles), and its index in the view in .w.
 
 // One tile of REC_TILE records of a view in depth order: gathers each one's
 // rect or tile mask, writes it and its first pair (relative to the view's
@@ -217,17 +214,11 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
 #pragma unroll
     for (int k = 0; k < REC_IPT; ++k) {
         const Rect q = tile_rect(uv[k].x, uv[k].y, rad[k], B, TX, TY);
-        uint32_t mlo = __float_as_uint(f2[k].y), mhi = __float_as_uint(f2[k].z);
-        const uint32_t w = (uint32_t)(q.x1 - q.x0), h = (uint32_t)(q.y1 - q.y0);
-        if ((mlo | mhi) == 0 && w <= 8 && h <= 8) {  // a whole rect that fits a mask
-            const uint32_t rows = 0x01010101u * ((1u << w) - 1u);
-            mlo = h >= 4 ? rows : rows & ((1u << (8 * h)) - 1u);
-            mhi = h <= 4 ? 0u : h == 8 ? rows : rows & ((1u << (8 * (h - 4))) - 1u);
-        }
-        const bool masked = (mlo | mhi) != 0;
-        out[k] = make_uint4((uint32_t)q.x0 | ((uint32_t)q.y0 << 16), masked ? mlo : w, masked ? mhi : h,
-                            (uint32_t)(r[k] - (uint32_t)(st.v * P)) | (masked ? 0u : kRectFlag));
-        cnt[k] = first + 32 * k < st.n ? (masked ? (uint32_t)(__popc(mlo) + __popc(mhi)) : w * h) : 0u;
+        const RecTiles t = pack_tiles((uint32_t)q.x0, (uint32_t)q.y0, (uint32_t)(q.x1 - q.x0), (uint32_t)(q.y1 - q.y0),
+                                      __float_as_uint(f2[k].y), __float_as_uint(f2[k].z), TX);
+        out[k] = make_uint4(t.corner, t.lo, t.hi, (uint32_t)(r[k] - (uint32_t)(st.v * P)));
+        cnt[k] = first + 32 * k >= st.n ? 0u
+               : t.lo ? (uint32_t)(__popc(t.lo) + __popc(t.hi)) : rect_width(t.hi, TX) * rect_height(t.hi, TX);
         const uint32_t inc = warp_incl_scan<uint32_t>(cnt[k], lane);
         ex[k] = run + inc - cnt[k];
         run += __shfl_sync(0xffffffffu, inc, 31);
@@ -266,7 +257,8 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
     for (int k = 0; k < REC_IPT; ++k) {
         if (cnt[k] == 0) continue;
         const uint32_t x0 = out[k].x & 0xffffu, y0 = out[k].x >> 16;
-        const bool masked = !(out[k].w & kRectFlag);
+        const bool masked = out[k].y != 0;
+        const uint32_t rw = rect_width(out[k].z, TX), rh = rect_height(out[k].z, TX);
         if (tk.npass == 1) {
             const uint32_t k0 = (y0 << tk.xbits) + x0;
             if (masked) {
@@ -278,8 +270,8 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
                 }
             } else {
 #pragma unroll 1
-                for (uint32_t y = 0; y < out[k].z; ++y) {
-                    const uint32_t a = k0 + (y << tk.xbits), e = a + out[k].y;
+                for (uint32_t y = 0; y < rh; ++y) {
+                    const uint32_t a = k0 + (y << tk.xbits), e = a + rw;
                     atomicAdd(&diff[a & dm], 1);
                     if (e <= dm) atomicAdd(&diff[e], -1);
                 }
@@ -289,7 +281,7 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
             auto cyc = [&](uint32_t n) { atomicAdd(&s_cycles, n); };
             const uint32_t a = y0 * (uint32_t)TX + x0;
             if (masked) count_linear_mask(a, TX, out[k].y, out[k].z, tk.width[0], add, cyc);
-            else count_linear_rect(a, TX, out[k].y, out[k].z, tk.width[0], add, cyc);
+            else count_linear_rect(a, TX, rw, rh, tk.width[0], add, cyc);
         } else if (masked) {
             // pairs of each of the mask's eight columns
             uint32_t any = out[k].y | out[k].z;
@@ -303,7 +295,7 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
             }
         } else {
             // columns x0 .. x0 + w - 1, each h times: cyclic through the digit's values
-            count_run(x0, out[k].y, out[k].z, tk.width[0], [&](uint32_t i, int n) { atomicAdd(&diff[i], n); },
+            count_run(x0, rw, rh, tk.width[0], [&](uint32_t i, int n) { atomicAdd(&diff[i], n); },
                       [&](uint32_t n) { atomicAdd(&s_cycles, n); });
         }
     }
@@ -369,8 +361,8 @@ struct SrcEmit {
             const uint32_t s = s_lo + (uint32_t)(on ? i0 + lane : 0);
             const uint4 c = rv[s];
             const int p0 = (int)(pv[s] - base);  // of the record's first pair in this tile's array (may be negative)
-            const bool whole = on && (c.w & kRectFlag) != 0;
-            const uint32_t g = rbase + (c.w & ~kRectFlag);
+            const bool whole = on && c.y == 0;
+            const uint32_t g = rbase + c.w;
             const uint32_t k0 = (c.x >> 16) * row + (c.x & 0xffffu);
             // the mask's two words in turn (most masks have no bit above the fourth tile row)
             int p = p0;
@@ -394,7 +386,8 @@ struct SrcEmit {
                 const int l = __ffs((int)todo) - 1;
                 todo &= todo - 1;
                 const int q0 = __shfl_sync(0xffffffffu, p0, l);
-                const uint32_t w = __shfl_sync(0xffffffffu, c.y, l), h = __shfl_sync(0xffffffffu, c.z, l);
+                const uint32_t size = __shfl_sync(0xffffffffu, c.z, l);
+                const uint32_t w = rect_width(size, tg.TX[st.v]), h = rect_height(size, tg.TX[st.v]);
                 const uint32_t kb = __shfl_sync(0xffffffffu, k0, l), gg = __shfl_sync(0xffffffffu, g, l);
                 const int a = q0 < 0 ? 0 : q0;
                 const long long end = (long long)q0 + (long long)w * h;

@@ -120,4 +120,47 @@ DG_HD void count_linear_rect(uint32_t key0, int TX, uint32_t w, uint32_t h, int 
     for (uint32_t y = 0; y < h; ++y) count_run(key0 + y * (uint32_t)TX, w, 1u, width, diff, cycles);
 }
 
+// A record's tiles in three words: the corner x0 | y0 << 16, then a mask of 8 x 8
+// tiles (a whole rect that fits one, too) or a larger rect's size.  A mask's low word
+// is never 0 (one with four empty rows starts four rows further down); with a low word
+// of 0 the last word is (w - 1) | (h - 1) << bits of a column, which is 31 bits at
+// most in a view's grid and 0 only where there are no tiles (1 x 1 is a mask).
+// The record's index keeps all 32 bits of its own word.
+struct RecTiles { uint32_t corner, lo, hi; };
+
+DG_HD int column_bits(int TX)
+{
+    int b = 0;
+#ifdef __CUDA_ARCH__
+    b = TX > 1 ? 32 - __clz(TX - 1) : 0;
+#else
+    while ((1ll << b) < TX) ++b;
+#endif
+    return b;
+}
+
+DG_HD RecTiles pack_tiles(uint32_t x0, uint32_t y0, uint32_t w, uint32_t h, uint32_t lo, uint32_t hi, int TX)
+{
+    if ((lo | hi) == 0 && w <= 8 && h <= 8) {
+        const uint32_t rows = 0x01010101u * ((1u << w) - 1u);
+        lo = h >= 4 ? rows : rows & ((1u << (8 * h)) - 1u);
+        hi = h <= 4 ? 0u : h == 8 ? rows : rows & ((1u << (8 * (h - 4))) - 1u);
+    }
+    RecTiles r;
+    if ((lo | hi) != 0) {
+        const bool down = lo == 0;
+        r.corner = x0 | ((y0 + (down ? 4u : 0u)) << 16);
+        r.lo = down ? hi : lo;
+        r.hi = down ? 0u : hi;
+    } else {
+        r.corner = x0 | (y0 << 16);
+        r.lo = 0;
+        r.hi = w == 0 || h == 0 ? 0u : (w - 1u) | ((h - 1u) << column_bits(TX));
+    }
+    return r;
+}
+// Size of a rect from its last word (with a low word of 0).
+DG_HD uint32_t rect_width(uint32_t hi, int TX) { return hi == 0 ? 0u : (hi & ((1u << column_bits(TX)) - 1u)) + 1u; }
+DG_HD uint32_t rect_height(uint32_t hi, int TX) { return hi == 0 ? 0u : (hi >> column_bits(TX)) + 1u; }
+
 }  // namespace dg

@@ -2,8 +2,8 @@
 for the host from the library's own header: over grids of every form (one digit,
 column and row digits, one column of more than 256 tiles, views whose columns and
 rows need more than 31 bits together) the digits cover the key, a key leads back
-to its tile, keys of one view are distinct, and the counts equal an enumeration
-of the record's tiles."""
+to its tile, keys of one view are distinct, the counts equal an enumeration
+of the record's tiles, and a record's three words lead back to its tiles."""
 from __future__ import annotations
 
 import os
@@ -69,6 +69,26 @@ int main(int argc, char** argv)
                     }
                     ++want[key(x0 + x, y0 + y) & dm];
                 }
+            {  // the record's words lead back to its tiles
+                const uint32_t rw = masked ? 9 : w, rh = masked ? 9 : h;
+                const RecTiles r = pack_tiles(x0 & 0xffffu, y0 & 0xffffu, rw, rh, lo, hi, TX);
+                const RecTiles none = pack_tiles(x0 & 0xffffu, y0 & 0xffffu, t & 2 ? 0 : w, t & 2 ? h : 0, 0, 0, TX);
+                if (none.lo || none.hi || rect_width(none.hi, TX) * rect_height(none.hi, TX)) return 8;
+                const uint32_t px = r.corner & 0xffffu, py = r.corner >> 16;
+                if (px != (x0 & 0xffffu)) return 9;
+                unsigned long long m = (unsigned long long)lo | ((unsigned long long)hi << 32);
+                if (!m && (rw > 8 || rh > 8)) {
+                    if (masked && (rw > (uint32_t)TX || rh > (uint32_t)TY)) continue;  // (9 x 9 stands in, where it fits)
+                    if (r.lo || rect_width(r.hi, TX) != rw || rect_height(r.hi, TX) != rh || py != (y0 & 0xffffu)) return 10;
+                } else {
+                    if (!m)
+                        for (uint32_t y = 0; y < rh; ++y)
+                            for (uint32_t x = 0; x < rw; ++x) m |= 1ull << (8 * y + x);
+                    const unsigned long long got = (unsigned long long)r.lo | ((unsigned long long)r.hi << 32);
+                    const uint32_t d = (py - y0) & 0xffffu;
+                    if (!r.lo || (d != 0 && d != 4) || (d ? m >> 32 : m) != got || (d && (uint32_t)m)) return 11;
+                }
+            }
             if (k.linear) {
                 if (masked) count_linear_mask(key(x0, y0), TX, lo, hi, k.width[0], add, full);
                 else count_linear_rect(key(x0, y0), TX, w, h, k.width[0], add, full);
