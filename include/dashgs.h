@@ -223,6 +223,15 @@ DG_API dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64_t P
 DG_API dg_status dg_lookback_probe(const uint64_t* look, int64_t tile, int32_t stride, int32_t digit,
                                    int32_t max_polls, uint64_t* sum, int32_t* err, dg_stream stream);
 
+/* The same for each form of the wait.  form 0: dg_lookback_probe's, 64-bit words
+ * (passes over segments of 2^30 items or more); 1: 32-bit words, the state in the
+ * top two bits and the count in the low 30 (all other passes); 2: 64-bit words of one
+ * column (stride 1) summed by a whole warp, 32 tiles a time (records and
+ * densification).  Also DG_ERR_ARG for another form, and for form 2 with stride > 1. */
+DG_API dg_status dg_lookback_probe_form(const void* look, int64_t tile, int32_t stride, int32_t digit,
+                                        int32_t max_polls, int32_t form, uint64_t* sum, int32_t* err,
+                                        dg_stream stream);
+
 /* Mixed-precision records for the render calls (opts->record = 1): each
  * float32 record of dg_project becomes 24 bytes, u and v float32 (pixel
  * positions need the full mantissa at 1600 px), conic A, B, C and opacity

@@ -24,7 +24,8 @@ DG_OK, DG_ERR_ARG, DG_ERR_CAPACITY, DG_ERR_TIMEOUT, DG_ERR_CUDA = 0, -1, -2, -3,
 
 MAX_VIEWS = 16
 EXPORTS = ("dg_last_error", "dg_abi_version", "dg_kernel_launches", "dg_project", "dg_bin_workspace_size", "dg_bin_count",
-           "dg_bin_sort", "dg_lookback_probe", "dg_render_workspace_size", "dg_render_fwd", "dg_render_bwd", "dg_pack_records", "dg_project_bwd", "dg_project_bwd_adam",
+           "dg_bin_sort", "dg_lookback_probe",
+           "dg_lookback_probe_form", "dg_render_workspace_size", "dg_render_fwd", "dg_render_bwd", "dg_pack_records", "dg_project_bwd", "dg_project_bwd_adam",
            "dg_project_bwd_adam_dev",
            "dg_loss_workspace_size", "dg_ssim_workspace_size", "dg_loss_l1_dssim",
            "dg_loss_l1", "dg_loss_l1_noalloc", "dg_adam_step", "dg_adam_hparams_fill", "dg_adam_step_dev",
@@ -133,6 +134,7 @@ _SIGS = {
     "dg_bin_count": ([_P, _P, _I64, _I32, _P, _SZ, _I64, _P, _P], _ST),
     "dg_bin_sort": ([_P, _P, _I64, _CAM, _I32, _I32, _P, _SZ, _I64, _P, _P, _P, _P], _ST),
     "dg_lookback_probe": ([_P, _I64, _I32, _I32, _I32, _P, _P, _P], _ST),
+    "dg_lookback_probe_form": ([_P, _I64, _I32, _I32, _I32, _I32, _P, _P, _P], _ST),
     "dg_render_workspace_size": ([_CAM, _I32, _OPT, _I64], _SZ),
     "dg_pack_records": ([_P, _I64, _P, _P], _ST),
     "dg_render_fwd": ([_P, _P, _P, _CAM, _I32, _OPT, _P, _P, _P, _P, _P, _P, _SZ, _P], _ST),
@@ -244,6 +246,11 @@ def dg_bin_workspace_size(P, n_views, M_cap) -> int:
 
 def dg_bin_count(depth, tiles, P, n_views, ws, ws_bytes, M_cap, M_out, stream=None):
     _check(_lib.dg_bin_count(_a(depth), _a(tiles), P, n_views, _a(ws), ws_bytes, M_cap, _a(M_out), _s(stream)))
+
+
+def dg_lookback_probe_form(look, tile, stride, digit, max_polls, form, sum_out, err_out, stream=None):
+    _check(_lib.dg_lookback_probe_form(_a(look), tile, stride, digit, max_polls, form, _a(sum_out), _a(err_out),
+                                       _s(stream)))
 
 
 def dg_lookback_probe(look, tile, stride, digit, max_polls, sum_out, err_out, stream=None):

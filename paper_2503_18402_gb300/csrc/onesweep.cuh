@@ -128,7 +128,8 @@ __device__ inline Word os_lookback(const Word* look, long long t, int stride, in
 
 // The same sum for one column of 64-bit words, taken by a whole warp, 32
 // predecessors a time; false when a wait gave up.
-__device__ inline bool os_lookback_warp(const uint64_t* look, long long t, uint64_t* out, int lane)
+__device__ inline bool os_lookback_warp(const uint64_t* look, long long t, uint64_t* out, int lane,
+                                        int max_polls = kLbPolls)
 {
     uint64_t& sum = *out;
     sum = 0;
@@ -149,7 +150,7 @@ __device__ inline bool os_lookback_warp(const uint64_t* look, long long t, uint6
         if (first < lim) return true;
         j -= use;
         if (use < 32) {
-            if (++polls > kLbPolls) return false;
+            if (++polls > max_polls) return false;
             __nanosleep(40);
         }
     }

@@ -664,20 +664,35 @@ extern "C" dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64
 
 // ------------------------------------------------------------ look-back probe
 namespace dg {
-__global__ void k_lookback_probe(const uint64_t* look, long long t, int stride, int d, int max_polls,
+// One warp: form 0 and 1 run in its first lane, form 2 in all of them.
+__global__ void k_lookback_probe(const void* look, long long t, int stride, int d, int max_polls, int form,
                                  uint64_t* sum, int* err)
 {
-    *err = 0;
+    const int lane = threadIdx.x;
+    if (lane == 0) *err = 0;
     __threadfence();
-    *sum = os_lookback(look, t, stride, d, err, max_polls);
+    __syncwarp();
+    if (form == 2) {
+        uint64_t s = 0;
+        const bool ok = os_lookback_warp((const uint64_t*)look, t, &s, lane, max_polls);
+        if (lane == 0) {
+            *sum = s;
+            if (!ok) atomicExch(err, DG_ERR_TIMEOUT);
+        }
+    } else if (lane == 0) {
+        *sum = form == 0 ? os_lookback((const uint64_t*)look, t, stride, d, err, max_polls)
+                         : (uint64_t)os_lookback((const uint32_t*)look, t, stride, d, err, max_polls);
+    }
 }
 }  // namespace dg
 
-extern "C" dg_status dg_lookback_probe(const uint64_t* look, int64_t tile, int32_t stride, int32_t digit,
-                                       int32_t max_polls, uint64_t* sum, int32_t* err, dg_stream stream)
+extern "C" dg_status dg_lookback_probe_form(const void* look, int64_t tile, int32_t stride, int32_t digit,
+                                            int32_t max_polls, int32_t form, uint64_t* sum, int32_t* err,
+                                            dg_stream stream)
 {
     if (!sum || !err || (tile > 0 && !look)) { dg_set_error("null buffer"); return DG_ERR_ARG; }
-    if (tile < 0 || stride < 1 || digit < 0 || digit >= stride) {
+    if (form < 0 || form > 2) { dg_set_error("bad look-back form %d", form); return DG_ERR_ARG; }
+    if (tile < 0 || stride < 1 || digit < 0 || digit >= stride || (form == 2 && stride != 1)) {
         dg_set_error("bad look-back probe: tile=%lld stride=%d digit=%d", (long long)tile, stride, digit);
         return DG_ERR_ARG;
     }
@@ -685,7 +700,13 @@ extern "C" dg_status dg_lookback_probe(const uint64_t* look, int64_t tile, int32
         dg_set_error("max_polls %d outside 0..%d", max_polls, dg::kLbPolls);
         return DG_ERR_ARG;
     }
-    dg::k_lookback_probe<<<1, 1, 0, (cudaStream_t)stream>>>(look, tile, stride, digit, max_polls, sum, err);
+    dg::k_lookback_probe<<<1, 32, 0, (cudaStream_t)stream>>>(look, tile, stride, digit, max_polls, form, sum, err);
     dg_note_launch();
     return dg_check_launch("lookback_probe");
+}
+
+extern "C" dg_status dg_lookback_probe(const uint64_t* look, int64_t tile, int32_t stride, int32_t digit,
+                                       int32_t max_polls, uint64_t* sum, int32_t* err, dg_stream stream)
+{
+    return dg_lookback_probe_form(look, tile, stride, digit, max_polls, 0, sum, err, stream);
 }
