@@ -136,17 +136,22 @@ struct SrcDepth {
 };
 
 // --------------------------------------------------------------- records in depth order
-constexpr int REC_IPT = 4;
-constexpr int REC_TILE = OS_THREADS * REC_IPT;
+// Records per thread: four, or one while that many records fill at most two blocks
+// per SM at four: a lone block's chain (gathers, counts, look-back) is most of the
+// kernel then (5k records on 120 tiles, phase 2: 38 -> 30 us; 334k records 36 with one
+// or four, 504k 46 with four and 54 with one).
+constexpr long long REC_SMALL_MAX = 152LL * 2 * OS_THREADS * 4;
+static int rec_ipt(long long n) { return n <= REC_SMALL_MAX ? 1 : 4; }
 
 // A record in depth order: its tiles (RecTiles), and its index in the view in .w.
 
-// One tile of REC_TILE records of a view in depth order: gathers each one's
+// One tile of a view's records in depth order: gathers each one's
 // rect or tile mask, writes it and its first pair (relative to the view's
 // pairs), the record holding each pair tile's first pair, and the counts of the
 // lowest tile digit.  Also clears the range table.  Positions fit 32 bits: with
 // more pairs than M_cap (< 2^32) nothing is written.  The prefix comes first and
 // the digits are counted while the first warp looks back.
+template <int REC_IPT>
 __global__ void __launch_bounds__(OS_THREADS)
 k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const uint32_t* __restrict__ order,
           long long P, int B, TileGrid tg, TileKey tk, Segs sg, const unsigned long long* __restrict__ npair,
@@ -154,6 +159,7 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
           uint4* __restrict__ rec, uint32_t* __restrict__ poff, uint32_t* __restrict__ bstart,
           uint2* __restrict__ ranges)
 {
+    constexpr int REC_TILE = OS_THREADS * REC_IPT;
     __shared__ int diff[OS_BINS];
     __shared__ uint32_t direct[OS_BINS];
     __shared__ uint32_t s_cycles;
@@ -259,24 +265,7 @@ k_records(const float4* __restrict__ feat, const int* __restrict__ radius, const
         const uint32_t x0 = out[k].x & 0xffffu, y0 = out[k].x >> 16;
         const bool masked = out[k].y != 0;
         const uint32_t rw = rect_width(out[k].z, TX), rh = rect_height(out[k].z, TX);
-        if (tk.npass == 1) {
-            const uint32_t k0 = (y0 << tk.xbits) + x0;
-            if (masked) {
-                unsigned long long mk = (unsigned long long)out[k].y | ((unsigned long long)out[k].z << 32);
-#pragma unroll 1
-                for (; mk; mk &= mk - 1) {
-                    const uint32_t b = (uint32_t)__ffsll((long long)mk) - 1u;
-                    atomicAdd(&direct[(k0 + ((b >> 3) << tk.xbits) + (b & 7u)) & dm], 1u);
-                }
-            } else {
-#pragma unroll 1
-                for (uint32_t y = 0; y < rh; ++y) {
-                    const uint32_t a = k0 + (y << tk.xbits), e = a + rw;
-                    atomicAdd(&diff[a & dm], 1);
-                    if (e <= dm) atomicAdd(&diff[e], -1);
-                }
-            }
-        } else if (tk.linear) {
+        if (tk.linear) {
             auto add = [&](uint32_t i, int n) { atomicAdd(&diff[i], n); };
             auto cyc = [&](uint32_t n) { atomicAdd(&s_cycles, n); };
             const uint32_t a = y0 * (uint32_t)TX + x0;
@@ -465,7 +454,7 @@ struct BinWs {
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Items per thread of a pass over at most n items, and the look-back word size.
-static int os_ipt(long long n) { return n <= OS_SMALL_MAX ? OS_IPT_SMALL : OS_IPT_BIG; }
+static int os_ipt(long long n, long long small_max) { return n <= small_max ? OS_IPT_SMALL : OS_IPT_BIG; }
 static size_t os_word(long long n) { return n < (1ll << 30) ? 4 : 8; }
 // Tiles of `views` segments holding n items together (each ends in a partial tile).
 static long long os_tiles(long long n, int views, int tile) { return n / tile + views; }
@@ -479,7 +468,7 @@ static BinWs bin_layout(char* base, long long P, int n_views, long long M_cap)
     w.M = (long long*)take(8);
     const size_t c1 = o;
     w.ctl1 = (BinCtl1*)take(sizeof(BinCtl1));
-    w.look1_pass = align256(os_word(N) * OS_BINS * (size_t)os_tiles(N, n_views, OS_THREADS * os_ipt(N)));
+    w.look1_pass = align256(os_word(N) * OS_BINS * (size_t)os_tiles(N, n_views, OS_THREADS * os_ipt(N, OS_SMALL_DEPTH)));
     w.look1 = take(4 * w.look1_pass);
     w.zero1 = o - c1;
     w.dk0 = (uint32_t*)take(4 * N); w.dv0 = (uint32_t*)take(4 * N);
@@ -488,10 +477,10 @@ static BinWs bin_layout(char* base, long long P, int n_views, long long M_cap)
     w.poff = (uint32_t*)take(4 * N);
     const size_t c2 = o;
     w.ctl2 = (BinCtl2*)take(sizeof(BinCtl2));
-    w.rlook = (uint64_t*)take(8 * os_tiles(N, n_views, REC_TILE));
+    w.rlook = (uint64_t*)take(8 * os_tiles(N, n_views, OS_THREADS * rec_ipt(N)));
     w.zero2_fixed = o - c2;
     // (from here on the offsets depend on M_cap)
-    const long long pt = os_tiles(M_cap, n_views, OS_THREADS * os_ipt(M_cap));
+    const long long pt = os_tiles(M_cap, n_views, OS_THREADS * os_ipt(M_cap, OS_SMALL_PAIRS));
     w.look2 = take(BIN_MAXPASS * align256(os_word(M_cap) * OS_BINS * pt));
     w.pk0 = (uint32_t*)take(4 * M_cap); w.pv0 = (uint32_t*)take(4 * M_cap);
     w.pk1 = (uint32_t*)take(4 * M_cap); w.pv1 = (uint32_t*)take(4 * M_cap);
@@ -502,9 +491,8 @@ static BinWs bin_layout(char* base, long long P, int n_views, long long M_cap)
 
 // One pass over at most n_max items; the kernel's form by the item count.
 template <int NB, class Src>
-static void os_pass(const Src& src, const Segs& sg, const OsPass& ps, long long n_max, cudaStream_t s)
+static void os_pass(const Src& src, const Segs& sg, const OsPass& ps, long long n_max, int ipt, cudaStream_t s)
 {
-    const int ipt = os_ipt(n_max);
     const int grid = (int)os_tiles(n_max, sg.V, OS_THREADS * ipt);
     if (ipt == OS_IPT_SMALL) k_os_pass<OS_IPT_SMALL, uint32_t, NB><<<grid, OS_THREADS, 0, s>>>(src, sg, ps);
     else if (os_word(n_max) == 4) k_os_pass<OS_IPT_BIG, uint32_t, NB><<<grid, OS_THREADS, 0, s>>>(src, sg, ps);
@@ -567,11 +555,12 @@ extern "C" dg_status dg_bin_count(const float* depth, const int32_t* tiles, int6
     };
     const Segs all{n_views, nullptr, P, P, LLONG_MAX, nullptr};
     const Segs vis{n_views, w.ctl1->nvis, 0, P, LLONG_MAX, nullptr};
-    os_pass<8>(SrcDepth{depth, tiles}, all, pass(0, w.dk1, w.dv1), N, s);
-    os_pass<8>(SrcKV{w.dk1, w.dv1}, vis, pass(1, w.dk0, w.dv0), N, s);
-    os_pass<8>(SrcKV{w.dk0, w.dv0}, vis, pass(2, w.dk1, w.dv1), N, s);
+    const int ipt = os_ipt(N, OS_SMALL_DEPTH);
+    os_pass<8>(SrcDepth{depth, tiles}, all, pass(0, w.dk1, w.dv1), N, ipt, s);
+    os_pass<8>(SrcKV{w.dk1, w.dv1}, vis, pass(1, w.dk0, w.dv0), N, ipt, s);
+    os_pass<8>(SrcKV{w.dk0, w.dv0}, vis, pass(2, w.dk1, w.dv1), N, ipt, s);
     // (the highest digit, sign and upper exponent bits, has few distinct values)
-    os_pass<0>(SrcKV{w.dk1, w.dv1}, vis, pass(3, nullptr, w.dv0), N, s);
+    os_pass<0>(SrcKV{w.dk1, w.dv1}, vis, pass(3, nullptr, w.dv0), N, ipt, s);
     return dg_check_launch("bin_count");
 }
 
@@ -610,7 +599,7 @@ extern "C" dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64
     if (n_tiles > (1ll << 30)) { dg_set_error("too many tiles"); return DG_ERR_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
     const TileKey tk = tile_key(tg);
-    const int ipt = os_ipt(M_cap);
+    const int ipt = os_ipt(M_cap, OS_SMALL_PAIRS);
     const int pair_tile = OS_THREADS * ipt;
     size_t look_at[BIN_MAXPASS + 1] = {0};
     for (int p = 0; p < tk.npass; ++p)
@@ -618,7 +607,8 @@ extern "C" dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64
     if (N > 0 && M_cap > 0) {
         cudaMemsetAsync(w.ctl2, 0, w.zero2_fixed + look_at[tk.npass], s);
         const Segs vis{n_views, w.ctl1->nvis, 0, P, LLONG_MAX, nullptr};
-        k_records<<<(int)os_tiles(N, n_views, REC_TILE), OS_THREADS, 0, s>>>(
+        auto records = rec_ipt(N) == 1 ? k_records<1> : k_records<4>;
+        records<<<(int)os_tiles(N, n_views, OS_THREADS * rec_ipt(N)), OS_THREADS, 0, s>>>(
             (const float4*)feat, radius, w.dv0, P, tile, tg, tk, vis, w.ctl1->npair, M_cap, pair_tile,
             &w.ctl1->err, w.ctl2, w.rlook, w.rec, w.poff, w.bstart, (uint2*)ranges);
         dg_note_launch();
@@ -647,8 +637,8 @@ extern "C" dg_status dg_bin_sort(const float* feat, const int32_t* radius, int64
                 ps.ranges = (uint2*)ranges;
                 for (int v = 0; v <= n_views; ++v) ps.toff[v] = tg.off[v];
             }
-            if (p == 0) os_pass<8>(SrcEmit{w.rec, w.poff, w.bstart, w.ctl1->nvis, P, tg, tk.linear, tk.xbits, w.ctl2}, pairs, ps, M_cap, s);
-            else os_pass<8>(SrcKV{ki, vi}, pairs, ps, M_cap, s);
+            if (p == 0) os_pass<8>(SrcEmit{w.rec, w.poff, w.bstart, w.ctl1->nvis, P, tg, tk.linear, tk.xbits, w.ctl2}, pairs, ps, M_cap, ipt, s);
+            else os_pass<8>(SrcKV{ki, vi}, pairs, ps, M_cap, ipt, s);
             ki = ko;
             vi = vo;
         }
