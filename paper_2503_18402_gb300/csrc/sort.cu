@@ -458,6 +458,19 @@ static int os_ipt(long long n, long long small_max) { return n <= small_max ? OS
 static size_t os_word(long long n) { return n < (1ll << 30) ? 4 : 8; }
 // Tiles of `views` segments holding n items together (each ends in a partial tile).
 static long long os_tiles(long long n, int views, int tile) { return n / tile + views; }
+// The largest number of such tiles for any count up to n, when counts up to small_max
+// take tiles of small_tile items: the layout's sizes do not shrink as counts grow, so
+// that a workspace laid out for more serves fewer.
+static long long os_tiles_upto(long long n, int views, long long small_max, int small_tile, int big_tile)
+{
+    const long long s = os_tiles(n < small_max ? n : small_max, views, small_tile);
+    const long long b = n > small_max ? os_tiles(n, views, big_tile) : 0;
+    return s > b ? s : b;
+}
+static long long pass_tiles_upto(long long n, int views, long long small_max)
+{
+    return os_tiles_upto(n, views, small_max, OS_THREADS * OS_IPT_SMALL, OS_THREADS * OS_IPT_BIG);
+}
 
 static BinWs bin_layout(char* base, long long P, int n_views, long long M_cap)
 {
@@ -469,18 +482,18 @@ static BinWs bin_layout(char* base, long long P, int n_views, long long M_cap)
     const size_t c1 = o;
     w.ctl1 = (BinCtl1*)take(sizeof(BinCtl1));
     w.look1_pass = align256(os_word(N) * OS_BINS * (size_t)os_tiles(N, n_views, OS_THREADS * os_ipt(N, OS_SMALL_DEPTH)));
-    w.look1 = take(4 * w.look1_pass);
-    w.zero1 = o - c1;
+    w.zero1 = o - c1 + 4 * w.look1_pass;
+    w.look1 = take(4 * align256(os_word(N) * OS_BINS * (size_t)pass_tiles_upto(N, n_views, OS_SMALL_DEPTH)));
     w.dk0 = (uint32_t*)take(4 * N); w.dv0 = (uint32_t*)take(4 * N);
     w.dk1 = (uint32_t*)take(4 * N); w.dv1 = (uint32_t*)take(4 * N);
     w.rec = (uint4*)take(16 * N);
     w.poff = (uint32_t*)take(4 * N);
     const size_t c2 = o;
     w.ctl2 = (BinCtl2*)take(sizeof(BinCtl2));
-    w.rlook = (uint64_t*)take(8 * os_tiles(N, n_views, OS_THREADS * rec_ipt(N)));
+    w.rlook = (uint64_t*)take(8 * os_tiles_upto(N, n_views, REC_SMALL_MAX, OS_THREADS, OS_THREADS * 4));
     w.zero2_fixed = o - c2;
     // (from here on the offsets depend on M_cap)
-    const long long pt = os_tiles(M_cap, n_views, OS_THREADS * os_ipt(M_cap, OS_SMALL_PAIRS));
+    const long long pt = pass_tiles_upto(M_cap, n_views, OS_SMALL_PAIRS);
     w.look2 = take(BIN_MAXPASS * align256(os_word(M_cap) * OS_BINS * pt));
     w.pk0 = (uint32_t*)take(4 * M_cap); w.pv0 = (uint32_t*)take(4 * M_cap);
     w.pk1 = (uint32_t*)take(4 * M_cap); w.pv1 = (uint32_t*)take(4 * M_cap);
