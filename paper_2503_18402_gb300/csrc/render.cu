@@ -273,69 +273,78 @@ __global__ void k_plan_items(const uint2* __restrict__ ranges, int n_tiles, RHdr
 
 // The whole plan in one block, for up to PLAN_TILES tiles: every automatic split
 // of 8x8 tiles (it happens below two tiles per resident CTA, 4864 here) and of
-// 16x16 tiles of common images.  A plan of a few tiles is launch-bound: the six
-// scan launches took 33 us from the first's start to the last's end at 16 tiles,
-// this one takes 5 us; 1k Gaussians at 64x64, forward and backward through the
-// autograd call: 513 -> 467 us.  Above it the scan's blocks read the ranges in parallel.
+// 16x16 tiles of common images.  A plan of a few tiles is launch-bound: the scans'
+// six launches take 30 us in a row.  Every item finds its tile by a search over the
+// tiles' first items, so all threads write items: written tile by tile by the warp
+// that holds the tile (consecutive tiles, so few warps worked), they took 21 us on 120
+// tiles and 37 on 351: the forward of 5 views of 85x62, 440 tiles, 80 -> 50 us.  Above
+// PLAN_TILES the scan's blocks read the ranges in parallel.
 constexpr int PLAN_THREADS = 1024;
-constexpr int PLAN_IPT = 8;
-constexpr int PLAN_TILES = PLAN_THREADS * PLAN_IPT;
+constexpr int PLAN_TILES = PLAN_THREADS * 8;
 __global__ void __launch_bounds__(PLAN_THREADS)
 k_plan_small(const uint2* __restrict__ ranges, int n_tiles, RHdr* hdr, SplitCfg cfg, int4* __restrict__ items,
              int4* __restrict__ sitems)
 {
     __shared__ uint64_t sm[33];
-    const int lane = threadIdx.x & 31;
-    const int t0 = threadIdx.x * PLAN_IPT;
-    long long len[PLAN_IPT];
+    __shared__ uint32_t s_off[PLAN_TILES];    // list length, then first item of each tile
+    __shared__ uint32_t s_slot[PLAN_THREADS]; // first chunk slot of each thread's tiles
+    const int tid = threadIdx.x;
     uint64_t acc = 0, tot;
-#pragma unroll
-    for (int i = 0; i < PLAN_IPT; ++i) {
-        len[i] = 0;
-        if (t0 + i < n_tiles) {
-            const uint2 r = ranges[t0 + i];
-            len[i] = (long long)(r.y - r.x);
-        }
-        acc += (uint64_t)len[i];
+    for (int t = tid; t < n_tiles; t += PLAN_THREADS) {
+        const uint2 r = ranges[t];
+        s_off[t] = r.y - r.x;
+        acc += r.y - r.x;
     }
     block_excl_scan<uint64_t>(acc, sm, &tot);
     const long long M = (long long)tot;
-    const int L = split_len(M, cfg);
-    // items (low 32 bits) and split chunks (high 32 bits) of the thread's tiles
-    int k[PLAN_IPT];
+    const uint32_t L = (uint32_t)split_len(M, cfg);
+    // a thread's tiles: 1 << sh consecutive ones
+    const int sh = n_tiles <= PLAN_THREADS ? 0 : n_tiles <= 2 * PLAN_THREADS ? 1 : n_tiles <= 4 * PLAN_THREADS ? 2 : 3;
+    const int t0 = tid << sh, t1 = min(n_tiles, t0 + (1 << sh));
+    auto chunks = [&](uint32_t len) { return len <= L ? 1u : (uint32_t)(((uint64_t)len + L - 1) / L); };
+    // items (low 32 bits) and split chunks (high 32 bits)
     uint64_t cnt = 0;
-#pragma unroll
-    for (int i = 0; i < PLAN_IPT; ++i) {
-        k[i] = t0 + i >= n_tiles ? 0 : len[i] <= L ? 1 : (int)((len[i] + L - 1) / L);
-        cnt += (uint64_t)k[i] | (k[i] > 1 ? (uint64_t)k[i] << 32 : 0);
+    for (int t = t0; t < t1; ++t) {
+        const uint32_t k = chunks(s_off[t]);
+        cnt += (uint64_t)k | (k > 1 ? (uint64_t)k << 32 : 0);
     }
-    uint64_t off = block_excl_scan<uint64_t>(cnt, sm, &tot);
-    if (threadIdx.x == 0) {
+    const uint64_t off = block_excl_scan<uint64_t>(cnt, sm, &tot);
+    const uint32_t n_items = (uint32_t)tot;
+    if (tid == 0) {
         hdr->M = M;
         hdr->totals = (long long)tot;
-        hdr->L = L;
-        hdr->n_items = (int)(tot & 0xffffffffull);
+        hdr->L = (int)L;
+        hdr->n_items = (int)n_items;
         hdr->n_slots = (int)(tot >> 32);
         hdr->planned = 1;
     }
-#pragma unroll
-    for (int i = 0; i < PLAN_IPT; ++i) {
-        const int io = (int)(off & 0xffffffffull), so = (int)(off >> 32);
-        if (k[i] == 1) items[io] = make_int4(t0 + i, 0, 1, -1);
-        // a split tile's chunks are written by the whole warp
-        uint32_t todo = __ballot_sync(0xffffffffu, k[i] > 1);
-        while (todo) {
-            const int l = __ffs((int)todo) - 1;
-            todo &= todo - 1;
-            const int kk = __shfl_sync(0xffffffffu, k[i], l), it = __shfl_sync(0xffffffffu, t0 + i, l);
-            const int io_l = __shfl_sync(0xffffffffu, io, l), so_l = __shfl_sync(0xffffffffu, so, l);
-            for (int c = lane; c < kk; c += 32) {
-                const int4 w = make_int4(it, c, kk, so_l);
-                items[io_l + c] = w;
-                sitems[so_l + c] = w;
-            }
+    s_slot[tid] = (uint32_t)(off >> 32);
+    uint32_t at = (uint32_t)off;
+    for (int t = t0; t < t1; ++t) {
+        const uint32_t k = chunks(s_off[t]);
+        s_off[t] = at;
+        at += k;
+    }
+    __syncthreads();
+    auto first = [&](int t) { return t < n_tiles ? s_off[t] : n_items; };
+    for (uint32_t i = tid; i < n_items; i += PLAN_THREADS) {
+        int lo = 0, hi = n_tiles - 1;  // the last tile whose first item is not behind i
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_off[mid] <= i) lo = mid; else hi = mid - 1;
         }
-        off += (uint64_t)k[i] | (k[i] > 1 ? (uint64_t)k[i] << 32 : 0);
+        const uint32_t f = s_off[lo], k = first(lo + 1) - f;
+        int4 w = make_int4(lo, (int)(i - f), (int)k, -1);
+        if (k > 1) {
+            uint32_t slot = s_slot[lo >> sh];
+            for (int t = (lo >> sh) << sh; t < lo; ++t) {
+                const uint32_t kt = first(t + 1) - s_off[t];
+                slot += kt > 1 ? kt : 0u;
+            }
+            w.w = (int)slot;
+            sitems[slot + (i - f)] = w;
+        }
+        items[i] = w;
     }
 }
 
