@@ -184,10 +184,12 @@ __device__ inline bool splat(const G3& g, const Cam& cam, float near_plane, floa
     return true;
 }
 
-struct ViewSet {
+struct Views {
     int n;
     Cam cam[DG_MAX_VIEWS];
     float campos[DG_MAX_VIEWS][3];
+};
+struct ViewSet : Views {
     int TX[DG_MAX_VIEWS], TY[DG_MAX_VIEWS];
 };
 
@@ -196,7 +198,7 @@ struct ViewSet {
 // every replay of a captured graph), the same set rebuilt from it in shared
 // memory (sizes and tile grids stay those of the host set).  Call with the
 // whole block; ends with a barrier when cdev is given.
-__device__ inline const ViewSet& block_views(const ViewSet& vs, const dg_camera* cdev, ViewSet* s_vs)
+__device__ inline const Views& block_views(const Views& vs, const dg_camera* cdev, Views* s_vs)
 {
     if (!cdev) return vs;
     for (int v = threadIdx.x; v < vs.n; v += blockDim.x) {
@@ -205,8 +207,6 @@ __device__ inline const ViewSet& block_views(const ViewSet& vs, const dg_camera*
         s_vs->cam[v].h = vs.cam[v].h;
         set_guard(s_vs->cam[v]);
         cam_centre(s_vs->cam[v], s_vs->campos[v]);
-        s_vs->TX[v] = vs.TX[v];
-        s_vs->TY[v] = vs.TY[v];
     }
     if (threadIdx.x == 0) s_vs->n = vs.n;
     __syncthreads();
@@ -295,8 +295,8 @@ k_project_fwd(const float* __restrict__ prm, long long stride, int P, ViewSet vs
               float near_plane, float eps2d, float mip2d, int tight, float4* __restrict__ feat, float* __restrict__ depth,
               int* __restrict__ radius, int* __restrict__ tiles, uint8_t* __restrict__ clampm)
 {
-    __shared__ ViewSet s_vs;
-    const ViewSet& vs = block_views(vs_host, cdev, &s_vs);
+    __shared__ Views s_vs;
+    const Views& vs = block_views(vs_host, cdev, &s_vs);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P) return;
     G3 g;
@@ -325,7 +325,7 @@ k_project_fwd(const float* __restrict__ prm, long long stride, int P, ViewSet vs
             const float vv = cam.fy * S.t[1] / tz + cam.cy;
             if (r3 <= kGuardPx && fabsf(u) <= kGuardPx && fabsf(vv) <= kGuardPx) {
                 const int rr = (int)ceilf(r3);
-                const Rect q = tile_rect(u, vv, rr, B, vs.TX[v], vs.TY[v]);
+                const Rect q = tile_rect(u, vv, rr, B, vs_host.TX[v], vs_host.TY[v]);
                 if (q.x0 < q.x1 && q.y0 < q.y1) {
                     float d0 = g.p[0] - vs.campos[v][0], d1 = g.p[1] - vs.campos[v][1], d2 = g.p[2] - vs.campos[v][2];
                     const float dinv = 1.f / sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
@@ -413,15 +413,23 @@ __device__ inline void stage_params(const float* __restrict__ prm, long long str
 // Adam for one view (five CTAs, measured 0.664 -> 0.648 ms at 2M Gaussians; six were
 // slower): the adjoint streams 0.5-1.5 kB per Gaussian, and the extra resident
 // warps hide more memory latency than the few spilled values cost.
-template <int NB, bool ADAM, bool SINGLE>
+// AHEAD: the radii of all views are loaded at once and a view's 2D gradients while the
+// view before it is worked on (one view: before its projection is formed again); else
+// each view's where they are used (load_ahead).  One view takes its gradients ahead when
+// they are stored (2M Gaussians, degree 3: 242 us, in place 254) and in place when fused
+// with Adam (477 against 495; degree 2 477 against 543).
+// Five CTAs of the fused one-view form leave 92 KB of an SM to the L1 cache while a CTA
+// takes at most 32,512 bytes: with 128 bytes more (tile grids beside the cameras) the
+// split of the two is the next one, and the kernel 4 to 8% slower.
+template <int NB, bool ADAM, bool SINGLE, bool AHEAD>
 __global__ void __launch_bounds__(128, ADAM && SINGLE ? 5 : 4)
-k_project_bwd(float* __restrict__ prm, long long stride, int P, ViewSet vs_host, const dg_camera* cdev,
+k_project_bwd(float* __restrict__ prm, long long stride, int P, Views vs_host, const dg_camera* cdev,
               float near_plane, float eps2d, float mip2d, const int* __restrict__ radius, const uint8_t* __restrict__ clampm,
               const float4* __restrict__ grad2d, float* __restrict__ grads, float* __restrict__ am,
               float* __restrict__ av, AdamHp hp_val, const AdamHp* __restrict__ hp_dev,
               const int* __restrict__ skip_if, int vec)
 {
-    __shared__ ViewSet s_vs;
+    __shared__ Views s_vs;
     __shared__ __align__(16) float s_g[ADAM ? DG_NPARAM : 1][128];  // ADAM: this CTA's gradients, for the row sweep
     __shared__ AdamHp s_hp;                            // ADAM: this step's hyper-parameters
     __shared__ AdamRowK s_rk[ADAM ? DG_NPARAM : 1];    // ADAM: per-row step and 1 / sqrt(1 - b2^t)
@@ -431,7 +439,7 @@ k_project_bwd(float* __restrict__ prm, long long stride, int P, ViewSet vs_host,
         for (int k = threadIdx.x; k < (int)(sizeof(AdamHp) / sizeof(float)); k += blockDim.x)
             ((float*)&s_hp)[k] = src[k];
     }
-    const ViewSet& vs = block_views(vs_host, cdev, &s_vs);
+    const Views& vs = block_views(vs_host, cdev, &s_vs);
     if (ADAM) {
         __syncthreads();  // s_hp complete (block_views has no barrier without device cameras)
         if (threadIdx.x < DG_NPARAM) s_rk[threadIdx.x] = adam_row(s_hp.lr[threadIdx.x], s_hp);
@@ -465,39 +473,16 @@ k_project_bwd(float* __restrict__ prm, long long stride, int P, ViewSet vs_host,
     #pragma unroll
         for (int k = 0; k < (SINGLE ? 1 : NB); ++k) dsh[k][0] = dsh[k][1] = dsh[k][2] = 0.f;
         bool any = false;
-        // the views that see the Gaussian (all radii loaded at once); a view's 2D
-        // gradients are loaded while the view before it is worked on, so a view
-        // waits for memory only when nothing was left to do meanwhile (SINGLE: one view)
-        uint32_t seen = 0;
-        if (SINGLE) {
-            seen = radius[i] != 0 ? 1u : 0u;
-        } else {
-#pragma unroll
-            for (int v = 0; v < DG_MAX_VIEWS; ++v)
-                if (v < vs.n) seen |= (radius[(size_t)v * P + i] != 0 ? 1u : 0u) << v;
-        }
-        float4 n0, n1;
-        float n2 = 0.f;
-        uint8_t ncm = 0;
-        auto fetch = [&](uint32_t left) {
-            if (!left) return;
-            const size_t r = (size_t)(__ffs((int)left) - 1) * P + i;
-            n0 = grad2d[3 * r];
-            n1 = grad2d[3 * r + 1];
-            n2 = grad2d[3 * r + 2].x;
-            ncm = clampm[r];
-        };
-        fetch(seen);
-        for (; seen; seen &= seen - 1) {
-            const int v = SINGLE ? 0 : __ffs((int)seen) - 1;
-            const float4 g0 = n0, g1 = n1;
-            const float g2x = n2;
-            const uint8_t cm = ncm;
-            if (!SINGLE) fetch(seen & (seen - 1));
+        // one view's share; load(g0, g1, g2, cm) gives its 2D gradients and colour clamp
+        auto add_view = [&](int v, auto load) {
             const Cam& cam = vs.cam[v];
             Splat S;
-            if (!splat(g, cam, near_plane, eps2d, mip2d, S)) continue;
+            if (!splat(g, cam, near_plane, eps2d, mip2d, S)) return;
             any = true;
+            float4 g0, g1;
+            float g2x;
+            uint8_t cm;
+            load(g0, g1, g2x, cm);
             const float dLu = g0.x, dLv = g0.y, dLA = g0.z, dLB = g0.w, dLC = g1.x;
             dop += g1.y * S.comp;  // record opacity = sigmoid * comp
             const float dcol[3] = {(cm & 1u) ? 0.f : g1.z, (cm & 2u) ? 0.f : g1.w, (cm & 4u) ? 0.f : g2x};
@@ -596,6 +581,46 @@ k_project_bwd(float* __restrict__ prm, long long stride, int P, ViewSet vs_host,
             // t = Rc p + t_c
     #pragma unroll
             for (int c = 0; c < 3; ++c) dp[c] += rc[c] * dt[0] + rc[3 + c] * dt[1] + rc[6 + c] * dt[2];
+        };
+        float4 n0, n1;
+        float n2 = 0.f;
+        uint8_t ncm = 0;
+        auto fetch = [&](int v) {
+            const size_t r = (size_t)v * P + i;
+            n0 = grad2d[3 * r];
+            n1 = grad2d[3 * r + 1];
+            n2 = grad2d[3 * r + 2].x;
+            ncm = clampm[r];
+        };
+        if (AHEAD) {
+            uint32_t seen = 0;
+            if (SINGLE) {
+                seen = radius[i] != 0 ? 1u : 0u;
+            } else {
+#pragma unroll
+                for (int v = 0; v < DG_MAX_VIEWS; ++v)
+                    if (v < vs.n) seen |= (radius[(size_t)v * P + i] != 0 ? 1u : 0u) << v;
+            }
+            auto next = [&](uint32_t left) {
+                if (left) fetch(__ffs((int)left) - 1);
+            };
+            next(seen);
+            for (; seen; seen &= seen - 1) {
+                const float4 c0 = n0, c1 = n1;
+                const float c2 = n2;
+                const uint8_t cc = ncm;
+                if (!SINGLE) next(seen & (seen - 1));
+                add_view(SINGLE ? 0 : __ffs((int)seen) - 1, [&](float4& g0, float4& g1, float& g2x, uint8_t& cm) {
+                    g0 = c0; g1 = c1; g2x = c2; cm = cc;
+                });
+            }
+        } else {
+            for (int v = 0; v < (SINGLE ? 1 : vs.n); ++v)
+                if (radius[(size_t)v * P + i] != 0)
+                    add_view(v, [&](float4& g0, float4& g1, float& g2x, uint8_t& cm) {
+                        fetch(v);
+                        g0 = n0; g1 = n1; g2x = n2; cm = ncm;
+                    });
         }
         if (!any) {
             for (int rr = 0; rr < DG_NPARAM; ++rr) put(rr, 0.f);
@@ -785,23 +810,42 @@ extern "C" dg_status dg_project(const float* params, int64_t stride, int64_t P, 
     return dg_check_launch("project_fwd");
 }
 
-template <bool ADAM, bool SINGLE>
+template <bool ADAM, bool SINGLE, bool AHEAD>
 static void launch_project_bwd(int nb, int blocks, int threads, cudaStream_t s, float* params, long long st, int P,
-                               const dg::ViewSet& vs, const dg_camera* cams_dev, const dg_raster_opts* opts,
+                               const dg_camera* cams, int n_views, const dg_camera* cams_dev, const dg_raster_opts* opts,
                                const int32_t* radius, const uint8_t* clamp, const float4* g2, float* grads, float* m,
                                float* v, const dg::AdamHp& hp, const dg::AdamHp* hp_dev, const int* skip_if)
 {
+    const dg::Views vs = make_views(cams, n_views, opts->tile);
     const float np = opts->near_plane, e2 = opts->eps2d, mp = opts->mip2d;
     // 16-byte row accesses in the Adam sweep: rows of params, m and v start on
     // 16-byte boundaries
     const int vec = ADAM && st % 4 == 0 && ((uintptr_t)params & 15u) == 0 && ((uintptr_t)m & 15u) == 0 &&
                     ((uintptr_t)v & 15u) == 0;
     switch (nb) {
-    case 1: dg::k_project_bwd<1, ADAM, SINGLE><<<blocks, threads, 0, s>>>(params, st, P, vs, cams_dev, np, e2, mp, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if, vec); break;
-    case 4: dg::k_project_bwd<4, ADAM, SINGLE><<<blocks, threads, 0, s>>>(params, st, P, vs, cams_dev, np, e2, mp, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if, vec); break;
-    case 9: dg::k_project_bwd<9, ADAM, SINGLE><<<blocks, threads, 0, s>>>(params, st, P, vs, cams_dev, np, e2, mp, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if, vec); break;
-    default: dg::k_project_bwd<16, ADAM, SINGLE><<<blocks, threads, 0, s>>>(params, st, P, vs, cams_dev, np, e2, mp, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if, vec); break;
+    case 1: dg::k_project_bwd<1, ADAM, SINGLE, AHEAD><<<blocks, threads, 0, s>>>(params, st, P, vs, cams_dev, np, e2, mp, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if, vec); break;
+    case 4: dg::k_project_bwd<4, ADAM, SINGLE, AHEAD><<<blocks, threads, 0, s>>>(params, st, P, vs, cams_dev, np, e2, mp, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if, vec); break;
+    case 9: dg::k_project_bwd<9, ADAM, SINGLE, AHEAD><<<blocks, threads, 0, s>>>(params, st, P, vs, cams_dev, np, e2, mp, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if, vec); break;
+    default: dg::k_project_bwd<16, ADAM, SINGLE, AHEAD><<<blocks, threads, 0, s>>>(params, st, P, vs, cams_dev, np, e2, mp, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if, vec); break;
     }
+}
+
+// Whether several views' 2D gradients are loaded one view ahead (AHEAD) or where they
+// are used.  Ahead, a view waits for memory only when nothing was left to do, but ten
+// registers are held across its work, and a few views have little to hide.  Measured
+// at 3k to 500k Gaussians and 2 to 16 views, time in place / time ahead:
+//   fused with Adam, degree 3: 0.99 to 1.01 at 2 to 4 views, 1.01 at 5, 1.02 to 1.06 at
+//   8, 1.07 at 16; degree 2: 0.91 to 0.98 at 5 and fewer, 0.98 to 1.02 at 8, 1.02 to 1.09
+//   at 16; degrees 1 and 0: 0.89 to 0.98 at 5 and fewer, 0.96 to 1.0 at 8, 1.02 at 16;
+//   gradients stored, degree 3: 0.9 to 0.99 below 2.4M records, 1.00 to 1.07 above at 8
+//   and 16 views; degree 2: 0.68 to 0.97; degree 1: 0.89 to 0.99 at 5 and fewer views or
+//   50k Gaussians, 1.0 to 1.03 above; degree 0: 0.96 to 1.0 at 50k Gaussians and fewer,
+//   1.01 to 1.13 from 150k on.
+static bool load_ahead(bool adam, int degree, int n_views, long long P)
+{
+    if (adam) return n_views >= (degree == 3 ? 6 : degree == 2 ? 8 : 12);
+    if (degree <= 1) return P >= 100000 && n_views >= (degree == 1 ? 8 : 2);
+    return degree == 3 && n_views >= 8 && P * n_views >= 2500000;
 }
 
 template <bool ADAM>
@@ -822,15 +866,19 @@ static dg_status project_bwd(float* params, int64_t stride, int64_t P, const dg_
         return DG_ERR_ARG;
     }
     if (((uintptr_t)grad2d) & 15u) { dg_set_error("grad2d must be 16-byte aligned"); return DG_ERR_ARG; }
-    const dg::ViewSet vs = make_views(cams, n_views, opts->tile);
     const int threads = 128;
     const int blocks = (int)((P + threads - 1) / threads);
     cudaStream_t s = (cudaStream_t)stream;
     const long long st = (long long)stride;
     const float4* g2 = (const float4*)grad2d;
     const int nb = opts->sh_degree == 0 ? 1 : opts->sh_degree == 1 ? 4 : opts->sh_degree == 2 ? 9 : 16;
-    if (n_views == 1) launch_project_bwd<ADAM, true>(nb, blocks, threads, s, params, st, (int)P, vs, cams_dev, opts, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if);
-    else launch_project_bwd<ADAM, false>(nb, blocks, threads, s, params, st, (int)P, vs, cams_dev, opts, radius, clamp, g2, grads, m, v, hp, hp_dev, skip_if);
+    auto go = [&](auto launch) {
+        launch(nb, blocks, threads, s, params, st, (int)P, cams, n_views, cams_dev, opts, radius, clamp, g2, grads, m,
+               v, hp, hp_dev, skip_if);
+    };
+    if (n_views == 1) go(launch_project_bwd<ADAM, true, !ADAM>);
+    else if (load_ahead(ADAM, opts->sh_degree, n_views, P)) go(launch_project_bwd<ADAM, false, true>);
+    else go(launch_project_bwd<ADAM, false, false>);
     dg_note_launch();
     return dg_check_launch(ADAM ? "project_bwd_adam" : "project_bwd");
 }
