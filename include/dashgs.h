@@ -321,9 +321,9 @@ DG_API dg_status dg_loss_l1(const float* img, const float* target, int64_t n, fl
  *      render layout); wh: host int32 [n_views][2] = (W_v, H_v).
  * Out: dL_dimg (same layout) = gradient of the mean over views of L_v;
  *      loss: device float32 [n_views + 1] = L_0 .. L_{n-1}, then the mean.
- * ws: dg_ssim_workspace_size(wh, n_views) bytes (36 bytes per pixel, the width
- * rounded up to strips of 128 columns, plus per-block sums); 0 is
- * returned for invalid sizes. */
+ * ws: dg_ssim_workspace_size(wh, n_views) bytes (36 bytes per pixel, the widths
+ * rounded up to strips of 128 columns, at most half as many again, plus per-block
+ * sums); 0 is returned for invalid sizes. */
 DG_API size_t dg_ssim_workspace_size(const int32_t* wh, int32_t n_views);
 DG_API dg_status dg_loss_l1_dssim(const float* img, const float* target, const int32_t* wh, int32_t n_views,
                                   float lambda, float* dL_dimg, float* loss, void* ws, size_t ws_bytes,

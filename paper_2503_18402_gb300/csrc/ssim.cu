@@ -11,8 +11,9 @@
 //   dS/dx(q) = F[dS/dmu_x](q) + 2 x(q) F[dS/da](q) + y(q) F[dS/dc](q),
 // F the same symmetric, zero-padded window.
 //
-// Two passes (k_ssim_fwd, k_ssim_bwd), each over strips of SS_W output columns
-// and segments of rows, a thread per two adjacent columns.  Going down the rows,
+// Two passes, over tiles (k_ssim_fwd_t, k_ssim_bwd_t) for small or narrow images, else
+// (k_ssim_fwd, k_ssim_bwd) over strips of SS_W output columns and segments of rows,
+// a thread per two adjacent columns.  Going down the rows,
 // two at a time are staged in shared memory; a thread forms the horizontal window
 // sums of its two columns from twelve staged inputs and feeds them to the vertical
 // windows, which it keeps as ten partial sums per column in registers (a new row
@@ -297,18 +298,18 @@ k_ssim_fwd(const float* __restrict__ img, const float* __restrict__ tgt, SViews 
 }
 
 // loss[v] = (1 - lam) l1_v + lam (1 - ssim_v); loss[n] = mean over views.  One
-// block: with one or two views four or two warps share a view, else each warp
-// takes every fourth one; a warp sums a fixed stride of its view's block sums in
+// block: NW warps shared evenly by the views, or, with more views than warps, each
+// warp taking every NW-th view; a warp sums a fixed stride of its view's block sums in
 // FP64, and the warps' and the views' sums are added in a fixed order, so the
 // result does not depend on timing.  It is the backward's first block: as a launch
 // of its own behind the backward it took 8 us for one view and 12 us for 16.
+template <int NW>
 __device__ void ssim_final(const float2* __restrict__ part, const SViews& sv, float lam, float* __restrict__ loss)
 {
-    constexpr int NW = SS_THREADS / 32;
     __shared__ double sm[2][DG_MAX_VIEWS][NW];
     __shared__ double lv_s[DG_MAX_VIEWS];
     const int nv = sv.n;
-    const int wpv = nv == 1 ? NW : nv == 2 ? NW / 2 : 1;  // warps per view
+    const int wpv = nv >= NW ? 1 : NW / nv;  // warps per view
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int v = w / wpv; v < nv; v += NW / wpv) {
         double s = 0.0, l = 0.0;
@@ -357,7 +358,7 @@ k_ssim_bwd(const float* __restrict__ img, const float* __restrict__ tgt, SViews 
     __shared__ __align__(16) float2 s_in[2][SS_ROWS][SS_E + 2];  // (dS/dmu_x, dS/da)
     __shared__ __align__(16) float s_c[2][SS_ROWS][SS_E + 2];    // dS/dc
     if (blockIdx.x == 0) {  // the losses, from the forward's block sums
-        ssim_final(part, sv, lam, loss);
+        ssim_final<SS_THREADS / 32>(part, sv, lam, loss);
         return;
     }
     const Blk b = decode(sv, blockIdx.x - 1);
@@ -469,73 +470,307 @@ k_ssim_bwd(const float* __restrict__ img, const float* __restrict__ tgt, SViews 
     }
 }
 
-}  // namespace
-}  // namespace dg
+// ------------------------------------------------------------ tiles
+// The same pass pair over 32x32 tiles of 256 threads: a tile and its halo are staged,
+// the horizontal and then the vertical window sums go through shared memory.  More
+// work per pixel than the strips, but a block is done in a fraction of a segment's
+// serial rounds and narrow images waste less of it (ssim_plan says which runs).  Maps in
+// the image's own layout [3 channels][H][W]; the gradient has the strips' bits (every
+// sum's taps in ascending order, the horizontal window first).
+constexpr int ST_T = 32;               // output tile edge
+constexpr int ST_E = ST_T + 2 * SS_R;  // staged edge (42)
+constexpr int ST_THREADS = 256;        // 32 x 8
 
-// Rows of a segment: the longest of 64, 32, 16 that gives at least five blocks
-// per SM, else 8: a segment repeats the window sums of ten rows.  (16 views of
-// 1237x822: 64 rows 0.615 ms, 128 0.635; one view, in a training step: 32 rows 8 us
-// less than 16.)
-static bool ssim_views(const int32_t* wh, int n_views, dg::SViews* sv, long long* nmap)
+__device__ __forceinline__ float tap(const Win& win, int k) { return win.w[k <= SS_R ? k : 2 * SS_R - k]; }
+
+// Stage plane[y0 - R .. y0 + T + R) x [x0 - R ..) into s (zero outside the image).
+// Thread t < 252 keeps column t % 42 and takes the rows t / 42 + 6 k (k < 7),
+// so its column test and offsets are formed once; all of its loads are issued
+// before its first shared store.
+constexpr int ST_SR = ST_THREADS / ST_E;  // staged rows per pass (6)
+static_assert(ST_E % ST_SR == 0, "the staged rows split evenly into passes");
+__device__ inline void stage(const float* __restrict__ plane, int W, int H, int x0, int y0, float (*s)[ST_E + 1])
 {
-    if (!wh) { dg_set_error("wh is null"); return false; }
-    if (n_views < 1 || n_views > DG_MAX_VIEWS) { dg_set_error("n_views %d outside 1..%d", n_views, DG_MAX_VIEWS); return false; }
-    sv->n = n_views;
-    for (int v = 0; v < n_views; ++v) {
-        const int W = wh[2 * v], H = wh[2 * v + 1];
-        if (W <= 0 || H <= 0 || W > (1 << 16) || H > (1 << 16)) { dg_set_error("view %d: image size %dx%d", v, W, H); return false; }
+    constexpr int NR = ST_E / ST_SR;
+    const int t = threadIdx.x;
+    if (t >= ST_SR * ST_E) return;
+    const int c = t % ST_E, r0 = t / ST_E;
+    const int x = x0 - SS_R + c;
+    const bool xok = x >= 0 && x < W;
+    const int ys = y0 - SS_R + r0;
+    float v[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+        const int y = ys + ST_SR * k;
+        v[k] = (xok && y >= 0 && y < H) ? plane[(size_t)y * W + x] : 0.f;
     }
-    for (int rows = 64;; rows /= 2) {
-        long long blocks = 0, pix = 0, map = 0;
-        sv->rows = rows;
-        for (int v = 0; v < n_views; ++v) {
-            const int W = wh[2 * v], H = wh[2 * v + 1];
-            sv->W[v] = W; sv->H[v] = H;
-            sv->TX[v] = (W + dg::SS_W - 1) / dg::SS_W;
-            sv->TY[v] = (H + rows - 1) / rows;
-            sv->boff[v] = (int)blocks;
-            sv->poff[v] = pix;
-            sv->moff[v] = map;
-            blocks += 3LL * sv->TX[v] * sv->TY[v];
-            pix += (long long)W * H;
-            map += 3LL * sv->TX[v] * H * dg::SS_W;
-            if (blocks >= (1LL << 31) - 1) { dg_set_error("images too large"); return false; }
+#pragma unroll
+    for (int k = 0; k < NR; ++k) s[r0 + ST_SR * k][c] = v[k];
+}
+
+// Work split of the two window passes: the horizontal pass gives each thread
+// ST_SL adjacent outputs of one staged row (one load per input, reused by the
+// ST_SL sums), the vertical pass ST_SL adjacent output rows of one column.
+constexpr int ST_SL = 4;
+static_assert((ST_THREADS / 32) * ST_SL == ST_T && ST_T / ST_SL == 8, "vertical: one warp per ST_SL rows; horizontal: 8 groups per row");
+
+__global__ void __launch_bounds__(ST_THREADS)
+k_ssim_fwd_t(const float* __restrict__ img, const float* __restrict__ tgt, SViews sv, Win win,
+           float* __restrict__ dm, float* __restrict__ da, float* __restrict__ dc, float2* __restrict__ part)
+{
+    __shared__ float sx[ST_E][ST_E + 1];
+    __shared__ float sy[ST_E][ST_E + 1];
+    // horizontal sums: mu_x, mu_y, a + b, c (S needs E[x^2] and E[y^2] only
+    // through their sum, so one window sum serves both)
+    __shared__ float hs[4][ST_E][ST_T];
+    __shared__ float red[2][ST_THREADS / 32];
+    const Blk b = decode(sv, blockIdx.x);
+    const int x0 = b.tx * ST_T, y0 = b.y0;
+    stage(img + b.plane, b.W, b.H, x0, y0, sx);
+    stage(tgt + b.plane, b.W, b.H, x0, y0, sy);
+    __syncthreads();
+    // (lanes: 8 groups of ST_SL columns x 4 rows per warp; banks all distinct)
+    for (int it = threadIdx.x; it < ST_E * (ST_T / ST_SL); it += ST_THREADS) {
+        const int r = it / (ST_T / ST_SL), c0 = (it % (ST_T / ST_SL)) * ST_SL;
+        float xv[ST_SL + 2 * SS_R], yv[ST_SL + 2 * SS_R];
+#pragma unroll
+        for (int q = 0; q < ST_SL + 2 * SS_R; ++q) { xv[q] = sx[r][c0 + q]; yv[q] = sy[r][c0 + q]; }
+#pragma unroll
+        for (int o = 0; o < ST_SL; ++o) {
+            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+            for (int k = 0; k <= 2 * SS_R; ++k) {
+                const float x = xv[o + k], y = yv[o + k], w = tap(win, k);
+                s0 = fmaf(w, x, s0);
+                s1 = fmaf(w, y, s1);
+                s2 = fmaf(w, fmaf(x, x, y * y), s2);
+                s3 = fmaf(w, x * y, s3);
+            }
+            hs[0][r][c0 + o] = s0; hs[1][r][c0 + o] = s1; hs[2][r][c0 + o] = s2;
+            hs[3][r][c0 + o] = s3;
         }
-        sv->boff[n_views] = (int)blocks;
-        *nmap = map;
-        if (blocks >= 5 * 152 || rows == 8) return true;
+    }
+    __syncthreads();
+    // vertical pass: lane = column, warp w = output rows ST_SL w .. ST_SL w + ST_SL - 1
+    const int c = threadIdx.x & 31, rb = (threadIdx.x >> 5) * ST_SL;
+    float st[4][ST_SL];  // window sums of the four statistics at this thread's outputs
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        float col[ST_SL + 2 * SS_R];
+#pragma unroll
+        for (int q = 0; q < ST_SL + 2 * SS_R; ++q) col[q] = hs[t][rb + q][c];
+#pragma unroll
+        for (int j = 0; j < ST_SL; ++j) {
+            float acc = 0.f;
+#pragma unroll
+            for (int k = 0; k <= 2 * SS_R; ++k) acc = fmaf(tap(win, k), col[j + k], acc);
+            st[t][j] = acc;
+        }
+    }
+    float ssum = 0.f, l1sum = 0.f;  // of 1 - S and |x - y|
+#pragma unroll
+    for (int j = 0; j < ST_SL; ++j) {
+        const int r = rb + j;
+        const int x = x0 + c, y = y0 + r;
+        if (x >= b.W || y >= b.H) continue;
+        const float mx = st[0][j], my = st[1][j], ab = st[2][j], cc = st[3][j];
+        const float A1 = 2.f * mx * my + kC1;
+        const float A2 = 2.f * (cc - mx * my) + kC2;
+        const float B1 = mx * mx + my * my + kC1;
+        const float B2 = (ab - mx * mx - my * my) + kC2;
+        const float inv = 1.f / (B1 * B2);
+        const float S = A1 * A2 * inv;
+        const size_t o = (size_t)b.plane + (size_t)y * b.W + x;
+        dm[o] = 2.f * my * (A2 - A1) * inv - 2.f * mx * S * (B2 - B1) * inv;
+        da[o] = -S * B1 * inv;
+        dc[o] = 2.f * A1 * inv;
+        ssum += 1.f - S;
+        l1sum += fabsf(sx[r + SS_R][c + SS_R] - sy[r + SS_R][c + SS_R]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        ssum += __shfl_xor_sync(0xffffffffu, ssum, o);
+        l1sum += __shfl_xor_sync(0xffffffffu, l1sum, o);
+    }
+    if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = ssum; red[1][threadIdx.x >> 5] = l1sum; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float s = 0.f, l = 0.f;
+        for (int w = 0; w < ST_THREADS / 32; ++w) { s += red[0][w]; l += red[1][w]; }
+        part[blockIdx.x] = make_float2(s, l);
     }
 }
 
-// Maps, then the block sums, with room for the shortest segments (so that a
-// workspace serves smaller images too) and for the maps' 16-byte alignment.
-static size_t ssim_map_bytes(long long nmap) { return ((size_t)3 * nmap * sizeof(float) + 255) & ~(size_t)255; }
-static size_t ssim_ws_bytes(const dg::SViews& sv, long long nmap)
+__global__ void __launch_bounds__(ST_THREADS, 4)
+k_ssim_bwd_t(const float* __restrict__ img, const float* __restrict__ tgt, SViews sv, Win win,
+           const float* __restrict__ dm, const float* __restrict__ da, const float* __restrict__ dc,
+           float lam, float* __restrict__ grad, const float2* __restrict__ part, float* __restrict__ loss)
 {
-    size_t blocks = 0;
-    for (int v = 0; v < sv.n; ++v) blocks += (size_t)3 * sv.TX[v] * ((sv.H[v] + 7) / 8);
-    return 16 + ssim_map_bytes(nmap) + sizeof(float2) * blocks;
+    __shared__ float s0[ST_E][ST_E + 1];
+    __shared__ float s1[ST_E][ST_E + 1];
+    __shared__ float s2[ST_E][ST_E + 1];
+    __shared__ float hs[3][ST_E][ST_T];
+    if (blockIdx.x == 0) {  // the losses, from the forward's block sums
+        ssim_final<ST_THREADS / 32>(part, sv, lam, loss);
+        return;
+    }
+    const Blk b = decode(sv, blockIdx.x - 1);
+    const int x0 = b.tx * ST_T, y0 = b.y0;
+    // this thread's outputs (column c, rows rb ..): their x and y are loaded
+    // first, so the loads' latency passes during the window sums
+    const int c = threadIdx.x & 31, rb = (threadIdx.x >> 5) * ST_SL;
+    float xo[ST_SL], yo[ST_SL];
+#pragma unroll
+    for (int j = 0; j < ST_SL; ++j) {
+        const int x = x0 + c, y = y0 + rb + j;
+        const bool in = x < b.W && y < b.H;
+        const size_t o = (size_t)b.plane + (size_t)(in ? y : 0) * b.W + (in ? x : 0);
+        xo[j] = in ? img[o] : 0.f;
+        yo[j] = in ? tgt[o] : 0.f;
+    }
+    stage(dm + b.plane, b.W, b.H, x0, y0, s0);
+    stage(da + b.plane, b.W, b.H, x0, y0, s1);
+    stage(dc + b.plane, b.W, b.H, x0, y0, s2);
+    __syncthreads();
+    for (int it = threadIdx.x; it < ST_E * (ST_T / ST_SL); it += ST_THREADS) {
+        const int r = it / (ST_T / ST_SL), c0 = (it % (ST_T / ST_SL)) * ST_SL;
+        float v0[ST_SL + 2 * SS_R], v1[ST_SL + 2 * SS_R], v2[ST_SL + 2 * SS_R];
+#pragma unroll
+        for (int q = 0; q < ST_SL + 2 * SS_R; ++q) { v0[q] = s0[r][c0 + q]; v1[q] = s1[r][c0 + q]; v2[q] = s2[r][c0 + q]; }
+#pragma unroll
+        for (int o = 0; o < ST_SL; ++o) {
+            float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+#pragma unroll
+            for (int k = 0; k <= 2 * SS_R; ++k) {
+                const float w = tap(win, k);
+                a0 = fmaf(w, v0[o + k], a0);
+                a1 = fmaf(w, v1[o + k], a1);
+                a2 = fmaf(w, v2[o + k], a2);
+            }
+            hs[0][r][c0 + o] = a0; hs[1][r][c0 + o] = a1; hs[2][r][c0 + o] = a2;
+        }
+    }
+    __syncthreads();
+    // d/dx of the mean over views of (1 - lam) mean|x - y| + lam (1 - mean S)
+    const float scale = 1.f / ((float)sv.n * 3.f * (float)b.W * (float)b.H);
+    float fs[3][ST_SL];  // filtered partial-derivative maps at this thread's outputs
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        float col[ST_SL + 2 * SS_R];
+#pragma unroll
+        for (int q = 0; q < ST_SL + 2 * SS_R; ++q) col[q] = hs[t][rb + q][c];
+#pragma unroll
+        for (int j = 0; j < ST_SL; ++j) {
+            float acc = 0.f;
+#pragma unroll
+            for (int k = 0; k <= 2 * SS_R; ++k) acc = fmaf(tap(win, k), col[j + k], acc);
+            fs[t][j] = acc;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < ST_SL; ++j) {
+        const int r = rb + j;
+        const int x = x0 + c, y = y0 + r;
+        if (x >= b.W || y >= b.H) continue;
+        const float f0 = fs[0][j], f1 = fs[1][j], f2 = fs[2][j];
+        const size_t o = (size_t)b.plane + (size_t)y * b.W + x;
+        const float xv = xo[j], yv = yo[j];
+        const float dS = f0 + 2.f * xv * f1 + yv * f2;
+        const float d = xv - yv;
+        const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
+        grad[o] = scale * ((1.f - lam) * sg - lam * dS);
+    }
+}
+
+}  // namespace
+}  // namespace dg
+
+// Strips of SS_W columns or tiles (see k_ssim_fwd_t), and the blocks of the call.
+struct SsimPlan {
+    dg::SViews sv;
+    bool tiles;
+    long long nmap;    // values of one map
+    size_t map_bytes;  // of the three maps, as the workspace holds them
+    size_t ws_bytes;
+};
+
+// Views cut into blocks of cols x rows pixels; maps in strips of map_cols columns (0: as
+// the image).
+static void ssim_blocks(const int32_t* wh, int n, int cols, int rows, int map_cols, SsimPlan* p)
+{
+    dg::SViews& sv = p->sv;
+    long long blocks = 0, pix = 0, map = 0;
+    sv.n = n;
+    sv.rows = rows;
+    for (int v = 0; v < n; ++v) {
+        const int W = wh[2 * v], H = wh[2 * v + 1];
+        sv.W[v] = W; sv.H[v] = H;
+        sv.TX[v] = (W + cols - 1) / cols;
+        sv.TY[v] = (H + rows - 1) / rows;
+        sv.boff[v] = (int)blocks;
+        sv.poff[v] = pix;
+        sv.moff[v] = map;
+        blocks += 3LL * sv.TX[v] * sv.TY[v];  // (at most 65536 x 65536 in each of 16 views)
+        pix += (long long)W * H;
+        map += 3LL * H * (map_cols ? sv.TX[v] * map_cols : W);
+    }
+    sv.boff[n] = (int)blocks;
+    p->nmap = map;
+}
+
+static bool ssim_plan(const int32_t* wh, int n_views, SsimPlan* p)
+{
+    if (!wh) { dg_set_error("wh is null"); return false; }
+    if (n_views < 1 || n_views > DG_MAX_VIEWS) { dg_set_error("n_views %d outside 1..%d", n_views, DG_MAX_VIEWS); return false; }
+    long long plain = 0, padded = 0, tile_blocks = 0;
+    for (int v = 0; v < n_views; ++v) {
+        const int W = wh[2 * v], H = wh[2 * v + 1];
+        if (W <= 0 || H <= 0 || W > (1 << 16) || H > (1 << 16)) { dg_set_error("view %d: image size %dx%d", v, W, H); return false; }
+        const long long strips = (W + dg::SS_W - 1) / dg::SS_W;
+        plain += (long long)W * H;
+        padded += strips * dg::SS_W * H;
+        tile_blocks += 3LL * ((W + dg::ST_T - 1) / dg::ST_T) * ((H + dg::ST_T - 1) / dg::ST_T);
+    }
+    // rows of a segment: 64 when that gives at least five blocks per SM, else 32: a
+    // segment repeats the window sums of ten rows.  (16 views of 1237x822: 64 rows
+    // 0.615 ms, 128 0.635; one view, in a training step: 32 rows 8 us less than 16.)
+    ssim_blocks(wh, n_views, dg::SS_W, 64, dg::SS_W, p);
+    if (p->sv.boff[n_views] < 5 * 152) ssim_blocks(wh, n_views, dg::SS_W, 32, dg::SS_W, p);
+    // Tiles while they are few (a strip's rounds are one chain: up to 2432 tiles, 16 per
+    // SM, 0.66 to 0.95 of the strips' time), and where the strips' padding or repeated
+    // rows cost more than the tiles' windows: a tile takes as long as about 11.5 rows of
+    // a strip (19 ns against 1.4 to 1.9).  One view of 1237x822: tiles 60 us, strips 52;
+    // 16 of 309x205 67 and 75, of 129x1000 146 and 172, of 16x3000 86 and 228, of 385x500
+    // 189 and 177.  (padded <= 1.5 plain holds the workspace's maps to that, too.)
+    long long strip_rows = 0;
+    for (int v = 0; v < n_views; ++v)
+        strip_rows += 3LL * p->sv.TX[v] * (p->sv.H[v] + 2 * dg::SS_R * p->sv.TY[v]);
+    p->tiles = padded * 2 > plain * 3 || tile_blocks <= 16 * 152 || 23 * tile_blocks < 2 * strip_rows;
+    if (p->tiles) ssim_blocks(wh, n_views, dg::ST_T, dg::ST_T, 0, p);
+    // the workspace: maps, then the block sums (of the tiles: never fewer than the strips'
+    // segments), so that it grows with every size and serves smaller images too; 16 bytes
+    // for the maps' alignment
+    const long long maps = padded * 2 <= plain * 3 ? padded : plain + (plain + 1) / 2;
+    p->map_bytes = ((size_t)3 * 3 * maps * sizeof(float) + 255) & ~(size_t)255;
+    p->ws_bytes = 16 + p->map_bytes + sizeof(float2) * (size_t)tile_blocks;
+    return true;
 }
 
 extern "C" size_t dg_ssim_workspace_size(const int32_t* wh, int32_t n_views)
 {
-    dg::SViews sv;
-    long long nmap = 0;
-    if (!ssim_views(wh, n_views, &sv, &nmap)) return 0;
-    return ssim_ws_bytes(sv, nmap);
+    SsimPlan p;
+    return ssim_plan(wh, n_views, &p) ? p.ws_bytes : 0;
 }
 
 extern "C" dg_status dg_loss_l1_dssim(const float* img, const float* target, const int32_t* wh, int32_t n_views,
                                       float lambda, float* dL_dimg, float* loss, void* ws, size_t ws_bytes,
                                       dg_stream stream)
 {
-    dg::SViews sv;
-    long long nmap = 0;
-    if (!ssim_views(wh, n_views, &sv, &nmap)) return DG_ERR_ARG;
+    SsimPlan p;
+    if (!ssim_plan(wh, n_views, &p)) return DG_ERR_ARG;
     if (!img || !target || !dL_dimg || !loss) { dg_set_error("null buffer"); return DG_ERR_ARG; }
     if (!(lambda >= 0.f && lambda <= 1.f)) { dg_set_error("lambda must be in [0, 1]"); return DG_ERR_ARG; }
-    const size_t need = ssim_ws_bytes(sv, nmap);
-    if (!ws || ws_bytes < need) { dg_set_error("ssim workspace missing or too small (%zu < %zu bytes)", ws_bytes, need); return DG_ERR_ARG; }
+    if (!ws || ws_bytes < p.ws_bytes) { dg_set_error("ssim workspace missing or too small (%zu < %zu bytes)", ws_bytes, p.ws_bytes); return DG_ERR_ARG; }
     dg::Win win;
     double sum = 0.0, w[2 * dg::SS_R + 1];
     for (int k = 0; k <= 2 * dg::SS_R; ++k) {
@@ -545,13 +780,18 @@ extern "C" dg_status dg_loss_l1_dssim(const float* img, const float* target, con
     }
     for (int k = 0; k <= dg::SS_R; ++k) win.w[k] = (float)(w[k] / sum);
     float* dm = (float*)(((uintptr_t)ws + 15) & ~(uintptr_t)15);
-    float* da = dm + nmap;
-    float* dc = da + nmap;
-    float2* part = (float2*)((char*)dm + ssim_map_bytes(nmap));
+    float* da = dm + p.nmap;
+    float* dc = da + p.nmap;
+    float2* part = (float2*)((char*)dm + p.map_bytes);
     cudaStream_t s = (cudaStream_t)stream;
-    const int nb = sv.boff[sv.n];
-    dg::k_ssim_fwd<<<nb, dg::SS_THREADS, 0, s>>>(img, target, sv, win, dm, da, dc, part);
-    dg::k_ssim_bwd<<<nb + 1, dg::SS_THREADS, 0, s>>>(img, target, sv, win, dm, da, dc, lambda, dL_dimg, part, loss);
+    const int nb = p.sv.boff[p.sv.n];
+    if (p.tiles) {
+        dg::k_ssim_fwd_t<<<nb, dg::ST_THREADS, 0, s>>>(img, target, p.sv, win, dm, da, dc, part);
+        dg::k_ssim_bwd_t<<<nb + 1, dg::ST_THREADS, 0, s>>>(img, target, p.sv, win, dm, da, dc, lambda, dL_dimg, part, loss);
+    } else {
+        dg::k_ssim_fwd<<<nb, dg::SS_THREADS, 0, s>>>(img, target, p.sv, win, dm, da, dc, part);
+        dg::k_ssim_bwd<<<nb + 1, dg::SS_THREADS, 0, s>>>(img, target, p.sv, win, dm, da, dc, lambda, dL_dimg, part, loss);
+    }
     dg_note_launch(2);
     return dg_check_launch("loss_l1_dssim");
 }

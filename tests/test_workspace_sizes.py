@@ -33,3 +33,16 @@ def test_binning_workspace_grows_with_every_count(capi):
     for P in counts[:-6]:
         sizes = [capi.dg_bin_workspace_size(P, v, 5 * lim + 1) for v in range(1, 17)]
         assert sizes == sorted(sizes)
+
+
+def test_loss_workspace_grows_with_every_size(capi):
+    import random
+    rng = random.Random(1)
+    for _ in range(2000):
+        big = [(rng.randint(1, 700), rng.randint(1, 700)) for _ in range(rng.choice([1, 1, 2, 3, 16]))]
+        small = [(rng.randint(1, w), rng.randint(1, h)) for w, h in big]
+        assert capi.dg_ssim_workspace_size(small) <= capi.dg_ssim_workspace_size(big), (small, big)
+    # narrow images: at most half as many map values again as pixels, and the block sums
+    for w in (1, 5, 33, 129):
+        n = w * 60000
+        assert capi.dg_ssim_workspace_size([(w, 60000)]) <= 36 * (n + n // 2 + 1) + 24 * (-(-w // 32)) * 1875 + 512
