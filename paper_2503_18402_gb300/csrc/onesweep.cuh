@@ -34,8 +34,8 @@
 // 33M pairs 1.16 against 1.23 ms for the whole binning with three; tiles of
 // 2048, 3072 or 5120 items 1.40, 1.23 and 1.37).  At 100k items a 1024-item tile
 // takes 6 us against 9 for 4096: the small tile is used while the items fill at
-// most three of them per SM in the depth order (334k items, four passes and counts,
-// 50 -> 45 us; 531k items 54 -> 60) and five, the most that are resident, in the
+// most two and a half of them per SM in the depth order (334k items, four passes and
+// counts, 50 -> 45 us; 467k items 53 -> 58, 531k 54 -> 60) and five, the most that are resident, in the
 // tile order, whose first pass also emits (330k to 690k pairs: 7 to 15 us less of
 // 45 to 64; 840k to 1.1M pairs 52 to 71 us, up to 9 more, with small tiles).
 #pragma once
@@ -51,7 +51,7 @@ constexpr int OS_WARPS = OS_THREADS / 32;
 constexpr int OS_BINS = 256;              // 8-bit digits, one thread per digit
 constexpr int OS_IPT_BIG = 16;
 constexpr int OS_IPT_SMALL = 4;
-constexpr long long OS_SMALL_DEPTH = 152LL * 3 * OS_THREADS * OS_IPT_SMALL;
+constexpr long long OS_SMALL_DEPTH = 152LL * 5 / 2 * OS_THREADS * OS_IPT_SMALL;
 constexpr long long OS_SMALL_PAIRS = 152LL * 5 * OS_THREADS * OS_IPT_SMALL;
 constexpr uint64_t kLbAgg = 1ull << 62;   // 64-bit word holding the tile's own total
 constexpr uint64_t kLbInc = 2ull << 62;   // 64-bit word holding the inclusive prefix

@@ -10,7 +10,7 @@ from tests.test_gpu_binning import test_lists_equal_the_numpy_construction as _c
 
 pytestmark = pytest.mark.gpu
 
-REC_LIMIT = 152 * 2 * 1024    # records: one per thread up to here, small depth tiles up to half as many again
+REC_LIMIT = 152 * 2 * 1024    # records: one per thread up to here; small depth tiles up to a quarter more
 
 
 @pytest.mark.parametrize("P,sizes,tile,tight", [
@@ -23,8 +23,8 @@ REC_LIMIT = 152 * 2 * 1024    # records: one per thread up to here, small depth 
     (256, [(100, 60)], 16, 0),
     (257, [(100, 60)], 16, 1),
     (REC_LIMIT, [(150, 100)], 16, 1),
-    (REC_LIMIT // 2, [(150, 100), (30, 20), (90, 60)], 16, 1),
-    (466945, [(50, 40)], 16, 0),             # one above the small depth tiles' limit
+    (REC_LIMIT * 5 // 16, [(150, 100), (30, 20), (90, 60), (50, 40)], 16, 1),  # at that limit
+    (REC_LIMIT * 5 // 4 + 1, [(50, 40)], 16, 0),                               # one above
 ])
 def test_small_grids_and_limits(P, sizes, tile, tight):
     _check(P, sizes, tile, tight)
