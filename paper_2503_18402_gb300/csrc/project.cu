@@ -198,7 +198,14 @@ struct ViewSet : Views {
 // every replay of a captured graph), the same set rebuilt from it in shared
 // memory (sizes and tile grids stay those of the host set).  Call with the
 // whole block; ends with a barrier when cdev is given.
-__device__ inline const Views& block_views(const Views& vs, const dg_camera* cdev, Views* s_vs)
+__device__ inline void copy_grids(const Views&, Views*, int) {}
+__device__ inline void copy_grids(const ViewSet& vs, ViewSet* s_vs, int v)
+{
+    s_vs->TX[v] = vs.TX[v];
+    s_vs->TY[v] = vs.TY[v];
+}
+template <class Set>
+__device__ inline const Set& block_views(const Set& vs, const dg_camera* cdev, Set* s_vs)
 {
     if (!cdev) return vs;
     for (int v = threadIdx.x; v < vs.n; v += blockDim.x) {
@@ -207,6 +214,7 @@ __device__ inline const Views& block_views(const Views& vs, const dg_camera* cde
         s_vs->cam[v].h = vs.cam[v].h;
         set_guard(s_vs->cam[v]);
         cam_centre(s_vs->cam[v], s_vs->campos[v]);
+        copy_grids(vs, s_vs, v);
     }
     if (threadIdx.x == 0) s_vs->n = vs.n;
     __syncthreads();
@@ -295,8 +303,8 @@ k_project_fwd(const float* __restrict__ prm, long long stride, int P, ViewSet vs
               float near_plane, float eps2d, float mip2d, int tight, float4* __restrict__ feat, float* __restrict__ depth,
               int* __restrict__ radius, int* __restrict__ tiles, uint8_t* __restrict__ clampm)
 {
-    __shared__ Views s_vs;
-    const Views& vs = block_views(vs_host, cdev, &s_vs);
+    __shared__ ViewSet s_vs;
+    const ViewSet& vs = block_views(vs_host, cdev, &s_vs);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P) return;
     G3 g;
@@ -325,7 +333,7 @@ k_project_fwd(const float* __restrict__ prm, long long stride, int P, ViewSet vs
             const float vv = cam.fy * S.t[1] / tz + cam.cy;
             if (r3 <= kGuardPx && fabsf(u) <= kGuardPx && fabsf(vv) <= kGuardPx) {
                 const int rr = (int)ceilf(r3);
-                const Rect q = tile_rect(u, vv, rr, B, vs_host.TX[v], vs_host.TY[v]);
+                const Rect q = tile_rect(u, vv, rr, B, vs.TX[v], vs.TY[v]);
                 if (q.x0 < q.x1 && q.y0 < q.y1) {
                     float d0 = g.p[0] - vs.campos[v][0], d1 = g.p[1] - vs.campos[v][1], d2 = g.p[2] - vs.campos[v][2];
                     const float dinv = 1.f / sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
@@ -834,8 +842,8 @@ static void launch_project_bwd(int nb, int blocks, int threads, cudaStream_t s, 
 // are used.  Ahead, a view waits for memory only when nothing was left to do, but ten
 // registers are held across its work, and a few views have little to hide.  Measured
 // at 3k to 500k Gaussians and 2 to 16 views, time in place / time ahead:
-//   fused with Adam, degree 3: 0.99 to 1.01 at 2 to 4 views, 1.01 at 5, 1.02 to 1.06 at
-//   8, 1.07 at 16; degree 2: 0.91 to 0.98 at 5 and fewer, 0.98 to 1.02 at 8, 1.02 to 1.09
+//   fused with Adam, degree 3: 0.98 to 1.0 at 2 to 4 views (1.0 to 1.03 at 3 and 4 and
+//   below 100k Gaussians), 1.0 to 1.03 at 5, 1.02 to 1.06 at 8, 1.07 at 16; degree 2: 0.91 to 0.98 at 5 and fewer, 0.98 to 1.02 at 8, 1.02 to 1.09
 //   at 16; degrees 1 and 0: 0.89 to 0.98 at 5 and fewer, 0.96 to 1.0 at 8, 1.02 at 16;
 //   gradients stored, degree 3: 0.9 to 0.99 below 2.4M records, 1.00 to 1.07 above at 8
 //   and 16 views; degree 2: 0.68 to 0.97; degree 1: 0.89 to 0.99 at 5 and fewer views or
@@ -843,7 +851,8 @@ static void launch_project_bwd(int nb, int blocks, int threads, cudaStream_t s, 
 //   1.01 to 1.13 from 150k on.
 static bool load_ahead(bool adam, int degree, int n_views, long long P)
 {
-    if (adam) return n_views >= (degree == 3 ? 6 : degree == 2 ? 8 : 12);
+    if (adam && degree == 3) return n_views >= (P < 100000 ? 3 : 6);
+    if (adam) return n_views >= (degree == 2 ? 8 : 12);
     if (degree <= 1) return P >= 100000 && n_views >= (degree == 1 ? 8 : 2);
     return degree == 3 && n_views >= 8 && P * n_views >= 2500000;
 }
