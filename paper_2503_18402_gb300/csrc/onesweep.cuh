@@ -32,12 +32,14 @@
 // votes' worth of instructions per digit bit became four instructions, and a
 // value is loaded only after its rank is known, so that four CTAs fit an SM (on
 // 33M pairs 1.16 against 1.23 ms for the whole binning with three; tiles of
-// 2048, 3072 or 5120 items 1.40, 1.23 and 1.37).  At 100k items a 1024-item tile
-// takes 6 us against 9 for 4096: the small tile is used while the items fill at
-// most two and a half of them per SM in the depth order (334k items, four passes and
-// counts, 50 -> 45 us; 467k items 53 -> 58, 531k 54 -> 60) and five, the most that are resident, in the
-// tile order, whose first pass also emits (330k to 690k pairs: 7 to 15 us less of
-// 45 to 64; 840k to 1.1M pairs 52 to 71 us, up to 9 more, with small tiles).
+// 2048, 3072 or 5120 items 1.40, 1.23 and 1.37).  At 64 registers for that the
+// 4096-item passes keep 72 to 104 bytes of a thread in local memory.  At 100k items a
+// 1024-item tile takes 6 us against 9 for 4096: the small tile is used while the
+// items fill at most two and a half of them per SM in the depth order (334k items,
+// four passes and counts, 50 -> 45 us; 467k items 53 -> 58, 531k 54 -> 60) and five,
+// the most that are resident, in the tile order, whose first pass also emits (330k
+// to 690k pairs: 7 to 15 us less of 45 to 64; 840k to 1.1M pairs 52 to 71 us, up to 9
+// more, with small tiles).
 #pragma once
 
 #include "scan.cuh"

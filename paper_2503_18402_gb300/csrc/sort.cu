@@ -19,7 +19,7 @@
 // drops the culled records, so the other three move only the visible ones.
 // Stage 2 (dg_bin_sort): one kernel walks the records in depth order, forms
 // each one's tile rect (16 bytes), scans their pair counts (look-back) and
-// counts the tile digits of all passes, a run of tiles at a time; the first
+// counts the lowest tile digit (each tile pass counts the next one); the first
 // tile pass emits its pairs straight into its ranking, so unsorted pairs never
 // reach memory; the last one extends the ranges of the tiles whose runs it
 // stages, so sorted keys are never stored.
@@ -440,7 +440,7 @@ struct BinWs {
     size_t look1_pass;                  // bytes of one pass
     size_t zero1;                       // bytes phase 1 clears from ctl1 on
     uint32_t *dk0, *dv0, *dk1, *dv1;   // depth sort, N each
-    uint4* rec;                         // records in depth order, N (over dk0, dk1 and two more words per record)
+    uint4* rec;                         // records in depth order, N
     uint32_t* poff;                     // N first pairs
     BinCtl2* ctl2;                      // phase 2 control block, then its look-back words
     uint64_t* rlook;                    // records scan

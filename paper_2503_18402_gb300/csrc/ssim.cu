@@ -32,9 +32,10 @@
 // 1237x822: 0.97 ms with 32x32 tiles (42x42 staged, both windows through shared
 // memory, a third of the threads idle in the horizontal pass's second round) and
 // a separate summing launch -> 0.615 ms, the gradient the same bits (six blocks per
-// SM, 160 registers; five 0.644, seven 0.618, eight 0.655).  The vertical window
-// first, four outputs per thread in the horizontal one, took 0.535 ms, but rounds
-// the gradient differently (3e-6 relative, no nearer to the exact one).
+// SM, 160 registers; five 0.644, seven 0.618, eight 0.655); 0.620 with
+// compensated sums.  The vertical window first, four outputs per thread in the
+// horizontal one, took 0.535 ms, but rounds the gradient differently (3e-6 relative,
+// no nearer to the exact one).
 #include <math.h>
 
 #include "common.cuh"
@@ -131,7 +132,7 @@ struct Col1 {
 // values, whose plain float32 sum carries their roundings one on another (1.9e-6 of a
 // constant |x - y|, against at most 11 roundings here).  1 - S is summed, not S: close
 // images lose nothing to sums near the pixel count (relative error of the loss at
-// |x - y| about 1e-3: 7.4e-7 -> 5.5e-7).  630 -> 636 us on 16 views of 1237x822.
+// |x - y| about 1e-3: 7.4e-7 -> 5.5e-7).  615 -> 620 us on 16 views of 1237x822.
 struct KSum2 {
     f32x2 s, c;  // c: what the sum lacks
     __device__ __forceinline__ void clear() { s = c = f2_pack(0.f, 0.f); }
